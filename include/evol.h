@@ -138,9 +138,9 @@ typedef struct {
     float alpha_u_min;         /* paper: 0 */
     int sph_scheme;            /* EVOL_SPH_LAGRANGIAN (0) or EVOL_SPH_STANDARD; the standard scheme
                                   needs 1 <= n_nei_sph (rounded) <= 335 */
-    int length_group;          /* particles per group walk of the length solves (they share one
-                                  tree walk listing the leaves near them): 0 = 8, or 1..32.
-                                  Changes cost, not the definition. */
+    int length_group;          /* particles that two warps of the length solves take together (1..32; the
+                                  warps of a block share one list of the leaves near them); 0: chosen
+                                  from the number of particles.  Changes cost, not the definition. */
 } evol_params;
 
 /* Outputs, caller order.  Any pointer may be NULL (not written). */
@@ -333,9 +333,9 @@ int evol_get_diagnostics(evol_ctx *ctx, double out[16]);
  *       pass (32 per entry or trip: interactions / slots is the fraction of busy lanes)
  *   [12] nodes popped by the force walk's groups, [13] of them tested lane by lane (neither
  *        accepted nor opened for the whole group), [14] leaves opened, [15] internal nodes opened
- *   length solves, eps at [16..19] and h at [20..23]: [+0] neighbour gathers from a group's leaf
- *        list, [+1] gathers by a particle's own tree walk, [+2] neighbour lists that overflowed,
- *        [+3] group leaf lists that overflowed
+ *   length solves, eps at [16..19] and h at [20..23]: [+0] neighbour gathers from a block's
+ *        candidates, [+1] gathers by a particle's own tree walk, [+2] neighbour lists that overflowed,
+ *        [+3] times a block's candidates did not fit
  *   [24] eps-solve and [25] h-solve Newton iterations (sum over particles)
  *   [26..31] zero */
 int evol_get_counters(evol_ctx *ctx, uint64_t out[32]);

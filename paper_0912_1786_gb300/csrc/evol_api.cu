@@ -13,7 +13,6 @@
 
 int evol_launch_pack(evol_ctx *c, const evol_particles *p, const evol_params *prm, int do_grav, int do_sph);
 int evol_launch_unpermute_ex(evol_ctx *c, const evol_particles *p, const evol_outputs *o, int what, int add_acc);
-int evol_lengths_warps_per_block();
 int evol_lengths_list_cap();
 int evol_launch_kick(evol_ctx *c, const evol_particles *p, const evol_params *prm, float half_dt, const float *ax,
                      const float *ay, const float *az, const float *dudt, const float *dalpha, const float *dalpha_u);
@@ -39,11 +38,11 @@ void free_all(evol_ctx *c)
     evol_dev &d = c->d;
     void *ptrs[] = {d.pos, d.vel, d.grav, d.hydro, d.snd, d.vah, d.orig, d.inv, d.divv_h, d.divv_e, d.mumax, d.dt, d.time, d.len_h, d.len_eps, d.nh, d.omega,
                     d.diss, d.curlv_h, d.vsig, d.lapu, d.dalpha, d.dalpha_u, d.tb, d.te, d.bact, d.pred_tau,
-                    d.pers, d.actf, d.acts, d.act, d.sg_acc, d.sg_front, d.sg_info, d.nbmin, d.bt, d.ewald,
+                    d.pers, d.actf, d.acts, d.act, d.gbase, d.glist, d.gpos, d.sg_acc, d.sg_front, d.sg_info, d.sg_rad, d.sg_stat, d.nbmin, d.bt, d.ewald,
                     d.zeta, d.rho, d.neps, d.ups, d.X, d.acc, d.dudt, d.keys_a, d.keys_b, d.vals_a, d.vals_b,
                     d.hist, d.lcp, d.cnt, d.base, d.scan_part, d.nbeg, d.nend, d.nlev, d.nnext, d.nparent,
                     d.nnch, d.narrive, d.nA, d.nB, d.nC, d.nQ0, d.nQ1, d.nM64, d.nC64, d.nQ64, d.nBmin,
-                    d.nBmax, d.nCoff, d.nI, d.nK0, d.nK1, d.wstack, d.cand_leaf, d.cand_mask, d.diag_part, d.diag, d.counters, d.err, d.nnodes,
+                    d.nBmax, d.nCoff, d.nI, d.nK0, d.nK1, d.wstack, d.diag_part, d.diag, d.counters, d.err, d.nnodes,
                     d.cube, d.fcube, d.bbox_part, d.hash3, d.cnt3, c->stage, c->kdk_acc, d.sys_off, d.sys_root, d.sys_sorted};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -295,8 +294,6 @@ int evol_create(evol_ctx **out, int64_t max_n, void *stream)
     c->sort_blocks = (max_n + 4095) / 4096;
     c->bbox_blocks = c->num_sms * 2;
     c->diag_blocks = c->num_sms * 2;
-    c->cand_cap = 0;
-    c->cand_slots = (int64_t)c->num_sms * 6 * evol_lengths_warps_per_block();   // length-solve warps
     c->wstack_slots = (int64_t)c->num_sms * 32;      // the walk and length grids use at most 32 warps per SM
     c->wstack_cap = WSTACK_CAP;
     c->wstack_lim = WSTACK_CAP;
@@ -314,10 +311,11 @@ int evol_create(evol_ctx **out, int64_t max_n, void *stream)
     rc |= dalloc(&d.dalpha, n); rc |= dalloc(&d.dalpha_u, n);
     rc |= dalloc(&d.tb, n); rc |= dalloc(&d.te, n); rc |= dalloc(&d.bact, n); rc |= dalloc(&d.pred_tau, n);
     rc |= dalloc(&d.pers, 7 * n); rc |= dalloc(&d.actf, n); rc |= dalloc(&d.acts, n + 1); rc |= dalloc(&d.act, n);
+    rc |= dalloc(&d.gbase, n + 1); rc |= dalloc(&d.glist, n); rc |= dalloc(&d.gpos, n);
     {
         const int64_t nsg = n / (32 * EVOL_SG_GROUPS) + 2;     // super-groups of the force walk
         rc |= dalloc(&d.sg_acc, nsg * EVOL_SG_ACAP); rc |= dalloc(&d.sg_front, nsg * EVOL_SG_FCAP);
-        rc |= dalloc(&d.sg_info, nsg);
+        rc |= dalloc(&d.sg_info, nsg); rc |= dalloc(&d.sg_rad, 4 * nsg); rc |= dalloc(&d.sg_stat, 2);
     }
     rc |= dalloc(&d.nbmin, n); rc |= dalloc(&d.bt, 8);
     rc |= dalloc(&d.ewald, (int64_t)EVOL_EWALD_M * EVOL_EWALD_M * EVOL_EWALD_M);
@@ -334,8 +332,6 @@ int evol_create(evol_ctx **out, int64_t max_n, void *stream)
     rc |= dalloc(&d.nBmin, nn); rc |= dalloc(&d.nBmax, nn); rc |= dalloc(&d.nCoff, nn); rc |= dalloc(&d.nI, nn);
     rc |= dalloc(&d.nK0, nn); rc |= dalloc(&d.nK1, nn);
     rc |= dalloc(&d.wstack, c->wstack_slots * c->wstack_cap);
-    rc |= dalloc(&d.cand_leaf, 1);                                      // unused
-    rc |= dalloc(&d.cand_mask, 1);
     rc |= dalloc(&d.diag_part, 16 * c->diag_blocks); rc |= dalloc(&d.diag, 16);
     rc |= dalloc(&d.counters, EVOL_NCOUNTERS); rc |= dalloc(&d.err, 1); rc |= dalloc(&d.nnodes, 1);
     c->nsys_cap = NSYS_CAP;

@@ -46,11 +46,17 @@ struct evol_dev {
     float *pred_tau;                // t_now - (tb + te)/2 (time units): prediction of v and u
     float *pers;                    // last evaluation: rho, Omega*, zeta, Upsilon, X, div v, |curl v| (7 x cap)
     int32_t *actf, *acts, *act;     // sorted: active flags, their exclusive scan (+ total), the list
+    // h solve of a set that is not all gas: gas particles before each sorted position (n + 1), the
+    // sorted position of each gas particle, and their positions and masses in that order
+    int32_t *gbase, *glist;
+    float4 *gpos;
     // force walk: per super-group (8 groups of 32 list entries) the nodes its bounds accept for all
     // its particles (EVOL_SG_ACAP each), the frontier its groups start from (EVOL_SG_FCAP each), and
     // their counts (-1: walk from the root)
     int32_t *sg_acc, *sg_front;
     int2 *sg_info;
+    float *sg_rad;           // length solves: search radius of each quarter of a super-group
+    unsigned long long *sg_stat;     // and the candidates of all super-groups, and their number
     unsigned *nbmin;                // sorted: smallest active-neighbour step (wake-up)
     unsigned long long *bt;         // [0] t_sys [1] t_next (ticks); [2..5] run counts
     float4 *ewald;                  // periodic gravity: correction table (f, g) for L = 1
@@ -78,9 +84,6 @@ struct evol_dev {
     int4 *nI;                           // walk copy: level | leaf << 8, next, begin, end
     int4 *nK0, *nK1;                    // child ids (up to 8, -1 padded) of internal nodes
     int2 *wstack;                       // per-warp traversal stacks of the force walk
-    // length solve scratch: per-lane (distance, mass) neighbour lists of every warp slot
-    int32_t *cand_leaf;
-    uint32_t *cand_mask;     // unused
     // reductions / counters
     double *diag_part;       // per-block partials of diagnostics
     double *diag;            // 16
@@ -106,7 +109,6 @@ struct evol_ctx {
     evol_dev d;
     int64_t sort_blocks;
     int64_t bbox_blocks;
-    int64_t cand_slots, cand_cap;
     int64_t wstack_slots, wstack_cap;
     int64_t wstack_lim;      // entries the walks may use per warp (<= wstack_cap)
     int64_t diag_blocks;
@@ -157,6 +159,8 @@ int evol_launch_integrator_step(evol_ctx *c, const evol_particles *p, const evol
                                 int stage);
 int evol_launch_bins(evol_ctx *c, const evol_particles *p, const evol_params *prm, const evol_bins *bp, int stage);
 int evol_launch_active_list(evol_ctx *c, int n);
+// Exclusive scan of n int32 (out may be in); write_total: out[n] receives the total.
+int evol_scan_i32(evol_ctx *c, int n, const int32_t *in, int32_t *out, int write_total);
 int evol_ewald_prepare(evol_ctx *c);
 
 #define EVOL_UNPERM_LENGTHS 1
@@ -183,6 +187,14 @@ static inline int evol_unperm_switches(const evol_params *prm)
 }
 // The Balsara factor (limiter, alpha source) needs div v and |curl v| from the h solve.
 static inline bool evol_needs_curl(const evol_params *prm) { return prm->sph && (prm->balsara || prm->variable_alpha); }
+
+// eps and h from one solve (mode 2 of the length solves): every particle is gas, so both count the same
+// neighbours, and the neighbour numbers are equal, so n L^3 = eta^3 is the same equation for both.
+static inline bool evol_shared_lengths(const evol_particles *p, const evol_params *prm)
+{
+    return prm->gravity && prm->adaptive_softening && prm->sph && p->n_gas == p->n &&
+           prm->n_nei_sph == prm->n_nei_grav && prm->sph_scheme == EVOL_SPH_LAGRANGIAN;
+}
 
 static inline int evol_cuda_ok(cudaError_t e) { return e == cudaSuccess ? EVOL_OK : EVOL_ECUDA; }
 
@@ -239,6 +251,55 @@ __device__ __forceinline__ float evol_tc_over_u(float u)
     return -0.75f * a * a / u;
 }
 
+// Packed two-wide FP32 arithmetic (add/mul/fma .rn.f32x2): one instruction computes the same
+// operation, rounded the same way, on two independent FP32 values held in a 64-bit register.
+// It halves the issue slots of the far-node loop and of the neighbour gathers.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk2(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v)
+{
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    (void)b;
+    return a;
+}
+__device__ __forceinline__ float hi2(f32x2 v)
+{
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    (void)a;
+    return b;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 // splitmix64 finaliser (Steele, Lea & Flood 2014), for interaction-set hashes in check mode.
 __device__ __forceinline__ unsigned long long evol_mix64(unsigned long long z)
 {
@@ -269,7 +330,7 @@ struct evol_kparams {
     float theta, G, gamma, alpha, beta;
     float eta_h, eta_e;
     int gravity, sph, adaptive, use_tc, periodic_mask, mixed;
-    float plen[3];
+    float plen[3], pinv[3];  // periodic lengths; 1/length (0 on an axis that is not periodic)
     int n, n_gas, leaf;
     int stack_cap;           // traversal-stack entries a warp may use
     int stack_stride;        // entries allocated per warp (>= stack_cap)
@@ -282,7 +343,8 @@ struct evol_kparams {
     // neighbour, the smallest step (ticks) of an active particle next to it (wake-up)
     int active, wake;
     int super;               // the force walk's groups start from their super-group's lists
-    int lsub;                // particles per group walk of the length solves (1..32)
+    int lists;               // the length solves' blocks take their leaves from super-group lists
+    int lsub;                // particles per warp of the length solves (1..32; 0: from their number)
     // periodic gravity (Ewald): cube side, 2 N / L for the table lookup, the table (L = 1)
     int ewald;
     float ewald_L, ewald_sc;

@@ -879,7 +879,7 @@ __global__ void k_zero_i32(const int32_t *__restrict__ nnodes, int32_t *a)
 // ---------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------
-static int scan_i32(evol_ctx *c, int n, const int32_t *in, int32_t *out, int write_total)
+int evol_scan_i32(evol_ctx *c, int n, const int32_t *in, int32_t *out, int write_total)
 {
     int nparts = (n + SC_TILE - 1) / SC_TILE;
     if (nparts < 1) nparts = 1;
@@ -913,7 +913,7 @@ int evol_launch_active_list(evol_ctx *c, int n)
     evol_dev &d = c->d;
     int tb = 256, gb = (n + tb - 1) / tb;
     k_active_flags<<<gb, tb, 0, c->stream>>>(n, d.orig, d.bact, d.actf);
-    int rc = scan_i32(c, n, d.actf, d.acts, 1);
+    int rc = evol_scan_i32(c, n, d.actf, d.acts, 1);
     if (rc) return rc;
     k_active_scatter<<<gb, tb, 0, c->stream>>>(n, d.actf, d.acts, d.act);
     return evol_cuda_ok(cudaGetLastError());
@@ -943,7 +943,7 @@ int evol_launch_build(evol_ctx *c, const evol_particles *p, const evol_params *p
     int32_t *va = d.vals_a, *vb = d.vals_b;
     for (int shift = 0; shift < 64; shift += 8) {
         k_rs_hist<<<rsb, RS_THREADS, 0, st>>>(n, ka, shift, (int32_t *)d.hist, rsb);
-        int rc = scan_i32(c, 256 * rsb, (int32_t *)d.hist, (int32_t *)d.hist, 0);
+        int rc = evol_scan_i32(c, 256 * rsb, (int32_t *)d.hist, (int32_t *)d.hist, 0);
         if (rc) return rc;
         k_rs_scatter<<<rsb, RS_THREADS, 0, st>>>(n, ka, va, kb, vb, shift, (int32_t *)d.hist, rsb);
         uint64_t *tk = ka; ka = kb; kb = tk;
@@ -956,7 +956,7 @@ int evol_launch_build(evol_ctx *c, const evol_particles *p, const evol_params *p
         ka = d.keys_b; kb = d.keys_a; va = d.vals_a; vb = d.vals_b;
         for (int shift = 0; (1ll << shift) < (long long)nsys; shift += 8) {
             k_rs_hist<<<rsb, RS_THREADS, 0, st>>>(n, ka, shift, (int32_t *)d.hist, rsb);
-            int rc = scan_i32(c, 256 * rsb, (int32_t *)d.hist, (int32_t *)d.hist, 0);
+            int rc = evol_scan_i32(c, 256 * rsb, (int32_t *)d.hist, (int32_t *)d.hist, 0);
             if (rc) return rc;
             k_rs_scatter<<<rsb, RS_THREADS, 0, st>>>(n, ka, va, kb, vb, shift, (int32_t *)d.hist, rsb);
             uint64_t *tk = ka; ka = kb; kb = tk;
@@ -971,7 +971,7 @@ int evol_launch_build(evol_ctx *c, const evol_particles *p, const evol_params *p
                                  c->pred_dt, c->kdk_acc, c->cap, c->pred_tau);
     k_lcp<<<gb, tb, 0, st>>>(n, d.keys_a, d.sys_off, nsys, d.lcp, d.sys_sorted);
     k_count<<<gb, tb, 0, st>>>(n, d.lcp, leaf, d.cnt);
-    int rc = scan_i32(c, n, d.cnt, d.base, 1);
+    int rc = evol_scan_i32(c, n, d.cnt, d.base, 1);
     if (rc) return rc;
     k_fill<<<gb, tb, 0, st>>>(n, d.keys_a, d.lcp, d.sys_off, d.sys_sorted, d.base, leaf, c->node_cap, d.nbeg, d.nend,
                               d.nlev, d.nnext, d.nnodes, d.err);

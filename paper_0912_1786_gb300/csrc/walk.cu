@@ -125,56 +125,6 @@ __device__ __forceinline__ int nth_bit(unsigned m, int k)
     return p;
 }
 
-// Packed two-wide FP32 arithmetic (add/mul/fma .rn.f32x2): one instruction computes the same
-// operation, rounded the same way, on two independent FP32 values held in a 64-bit register.
-// The far-node loop evaluates two accepted nodes per lane with it, which halves the issue slots
-// its arithmetic needs.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pk2(float lo, float hi)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float lo2(f32x2 v)
-{
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    (void)b;
-    return a;
-}
-__device__ __forceinline__ float hi2(f32x2 v)
-{
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    (void)a;
-    return b;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 // Periodic gravity: trilinear interpolation in the Ewald table (Sect. 4.3).  f is odd in its own
 // coordinate and even in the others, g is even, so the table holds the octant [0, L/2]^3 only; the
 // four components are interpolated as two packed pairs, (f_x, f_y) and (f_z, g), and the caller
