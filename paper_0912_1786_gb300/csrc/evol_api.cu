@@ -158,10 +158,11 @@ int record_phase(evol_ctx *c, int k, evol_particles *p, const evol_params *prm, 
         rc = evol_launch_build(c, p, prm);
         break;
     case 1:
-        if (grav && prm->adaptive_softening) rc = evol_launch_lengths(c, p, prm, 1);
+        if (grav && prm->adaptive_softening)
+            rc = evol_launch_lengths(c, p, prm, evol_shared_lengths(p, prm) ? 2 : 1);
         break;
     case 2:
-        if (sph) rc = evol_launch_lengths(c, p, prm, 0);
+        if (sph && !evol_shared_lengths(p, prm)) rc = evol_launch_lengths(c, p, prm, 0);
         if (!rc) rc = evol_launch_pack(c, p, prm, grav, sph);
         if (!rc) rc = evol_launch_node_lengths(c, prm, (int)p->n_gas);
         break;
@@ -839,8 +840,9 @@ int evol_run_bins(evol_ctx *c, evol_particles *p, const evol_params *prm, const 
                 // solves and walk over the active list; the inactive keep their last evaluation
                 c->bins_active = 1;
                 c->bins_wake = wake;
-                if (!prc && grav && prm->adaptive_softening) prc = evol_launch_lengths(c, p, prm, 1);
-                if (!prc && sph) prc = evol_launch_lengths(c, p, prm, 0);
+                const bool shared = evol_shared_lengths(p, prm);
+                if (!prc && grav && prm->adaptive_softening) prc = evol_launch_lengths(c, p, prm, shared ? 2 : 1);
+                if (!prc && sph && !shared) prc = evol_launch_lengths(c, p, prm, 0);
                 if (!prc) prc = evol_launch_bins(c, p, prm, bp, 2);
                 if (!prc) prc = evol_launch_pack(c, p, prm, grav, sph);
                 if (!prc) prc = evol_launch_node_lengths(c, prm, (int)ng);
