@@ -39,29 +39,38 @@ constexpr int SG_GROUPS = EVOL_SG_GROUPS;   // groups per super-group (see k_sup
 
 constexpr float TAU = 1e-5f;      // safety margin of the group-level bounds
 
+// One warp's shared memory: one base address for all of it, every array at a constant offset.
 struct WalkSmem {
-    float4 bA[WK_WARPS][32];      // popped batch: com, ropen^2
-    float4 bB[WK_WARPS][32];      // box centre, 2 hmax
-    float4 bC[WK_WARPS][32];      // box half widths, 2 epsmax
-    int far_id[WK_WARPS][FARCAP];
-    unsigned far_mask[WK_WARPS][FARCAP];
+    float4 bB[32];      // box centre, 2 hmax
+    float4 bC[32];      // box half widths, 2 epsmax
+    int near_j[NEARCAP];
+    unsigned near_mask[NEARCAP];       // lanes that opened the entry's leaf, less its own lane
+    // near entries in pairs for the two-wide first pass: component c of entry 2q + k sits at
+    // npair[q][2c + k], c = x, y, z, m, E = (2 eps)^2, H = (2 h)^2 (-1: not gas)
+    __align__(16) float npair[NEARCAP / 2][12];
+    float4 ng[NEARCAP];
+    float4 nh[NEARCAP];
+    float4 ns[NEARCAP];
+    float4 gbox[3];     // group bounds: centre, 0 | half widths, 0 | emax, emin, hmax, hmin
+    unsigned wc[8];     // per-group work counts kept by lane 0 (see the end of k_walk)
+    float mum[32];      // largest |mu_ij| of each lane's particle (viscosity)
+    int gs[32];         // active list: the sorted position of each lane's particle
+    unsigned gself[32]; // active list: the lane whose particle is a leaf chunk's entry
+};
+
+// The far list, and the popped batch's centres of mass: only the gravity walks hold them.
+template <bool GRAV>
+struct FarSmem {
+    float4 bA[32];                // popped batch: com, ropen^2
+    int far_id[FARCAP];
+    unsigned far_mask[FARCAP];
     // far nodes in pairs for the packed two-wide evaluation: for the pair of entries (2p, 2p + 1),
     // component c of entry 2p + k sits at fpair[p][2c + k], c = x, y, z, -M, Qxx, Qyy, Qzz, Qxy,
     // Qxz, Qyz (centre of mass, mass and traceless quadrupole)
-    __align__(16) float fpair[WK_WARPS][FARCAP / 2][20];
-    int near_j[WK_WARPS][NEARCAP];
-    unsigned near_mask[WK_WARPS][NEARCAP];       // lanes that opened the entry's leaf, less its own lane
-    // near entries in pairs for the two-wide first pass: component c of entry 2q + k sits at
-    // npair[q][2c + k], c = x, y, z, m, E = (2 eps)^2, H = (2 h)^2 (-1: not gas)
-    __align__(16) float npair[WK_WARPS][NEARCAP / 2][12];
-    float4 ng[WK_WARPS][NEARCAP];
-    float4 nh[WK_WARPS][NEARCAP];
-    float4 ns[WK_WARPS][NEARCAP];
-    float4 gbox[WK_WARPS][3];     // group bounds: centre, 0 | half widths, 0 | emax, emin, hmax, hmin
-    unsigned wc[WK_WARPS][8];     // per-group work counts kept by lane 0 (see the end of k_walk)
-    float mum[WK_WARPS][32];      // largest |mu_ij| of each lane's particle (viscosity)
-    int gs[WK_WARPS][32];         // active list: the sorted position of each lane's particle
-    unsigned gself[WK_WARPS][32]; // active list: the lane whose particle is a leaf chunk's entry
+    __align__(16) float fpair[FARCAP / 2][20];
+};
+template <>
+struct FarSmem<false> {
 };
 
 // The kernel functions of the pair loop in a division-free form: each takes u and iu = 1/u (iu is
@@ -182,7 +191,7 @@ template <bool MIXED>
 struct MixSmem {
     // [0, 4): compensation terms of ax, ay, az, pot; [4, 8): the running totals, parked here while
     // the pair loop sums its flush block in their registers
-    float c[WK_WARPS][8][32];
+    float c[8][32];
 };
 template <>
 struct MixSmem<false> {
@@ -192,9 +201,9 @@ struct MixSmem<false> {
 // each lane's running v^sig maximum and Brookshaw sum: only the DISS variants hold them.
 template <bool DISS>
 struct DissSmem {
-    float4 nd[WK_WARPS][NEARCAP];
-    float vs[WK_WARPS][32];
-    float lap[WK_WARPS][32];
+    float4 nd[NEARCAP];
+    float vs[32];
+    float lap[32];
 };
 template <>
 struct DissSmem<false> {
@@ -204,28 +213,31 @@ struct DissSmem<false> {
 // evaluates the pair (integer sums, so the order does not matter).
 template <bool CHECK>
 struct CheckSmem {
-    int cs[WK_WARPS][32];
-    unsigned long long hs[WK_WARPS][32];
-    int norig[WK_WARPS][NEARCAP];                 // original index of each near entry
+    int cs[32];
+    unsigned long long hs[32];
+    int norig[NEARCAP];                 // original index of each near entry
 };
 template <>
 struct CheckSmem<false> {
 };
 
 // Register budgets, chosen so that no variant spills to local memory: the gravity + SPH walk (the
-// production form, plain or mixed) and the SPH-only walk fit five blocks per SM (at most 102
-// registers), the walks with the dissipation variants (DISS) and the plain gravity-only periodic
-// (EWALD) walk four (128 registers), the other gravity-only, periodic and mixed DISS walks three;
-// the check-mode variants one.
+// production form, plain or mixed) fits five blocks per SM (at most 102 registers), the SPH-only walk, which
+// holds no far list, six (80); the walks with the dissipation variants (DISS), the plain gravity-only walk
+// and the plain gravity-only periodic one (EWALD) four (128 registers); the other periodic and mixed DISS
+// walks three; the check-mode variants one.  What made room: one base address for all of a warp's shared
+// memory, and a first pair pass that is not unrolled (gravity only, 2^20 Plummer particles: three blocks and
+// 6.7 ms before, four and 5.9 ms now; SPH only, 1.05 M-particle shock tube: five blocks and 3.6 ms before,
+// six and 2.8 ms now).
 template <bool GRAV, bool SPH, bool MIXED, bool CHECK, bool DISS, bool EWALD>
-__global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIXED) ? 4 : (EWALD || (GRAV && !SPH) || (MIXED && DISS)) ? 3 : DISS ? 4 : EVOL_WALK_MINB) k_walk(evol_dev d, evol_kparams kp, unsigned long long *queue)
+__global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIXED) ? 4 : (EWALD || (MIXED && DISS)) ? 3 : DISS || !SPH ? 4 : !GRAV ? 6 : EVOL_WALK_MINB) k_walk(evol_dev d, evol_kparams kp, unsigned long long *queue)
 {
-    __shared__ WalkSmem sm;
-    __shared__ DissSmem<DISS> ds;
-    __shared__ CheckSmem<CHECK> cks;
-    __shared__ MixSmem<MIXED> mx;
+    struct WarpSmem : WalkSmem, FarSmem<GRAV>, DissSmem<DISS>, CheckSmem<CHECK>, MixSmem<MIXED> {
+    };
+    __shared__ WarpSmem smem[WK_WARPS];
     const int lane = threadIdx.x & 31;
     const int w = threadIdx.x >> 5;
+    WarpSmem &sm = smem[w];
     const int n = kp.n;
     // individual time steps: groups of 32 consecutive entries of the active list
     const int nlist = kp.active ? d.acts[n] : n;
@@ -249,7 +261,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         const int s = kp.active ? (valid ? d.act[e] : 0) : e;
         const float4 pi = valid ? d.pos[s] : make_float4(0.f, 0.f, 0.f, 0.f);
         // the group's sorted positions, for the self test of the near list (active list only)
-        if (kp.active) sm.gs[w][lane] = valid ? s : -1;
+        if (kp.active) sm.gs[lane] = valid ? s : -1;
         // this lane's hydro operands (v, P/rho^2, c, rho, 1/h, zeta/Omega*) are read where they are
         // used, in the SPH pass, which keeps them out of the traversal's live registers
         const float4 g0 = valid ? d.grav[s] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -270,20 +282,20 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         // per-group counts kept by lane 0 in shared memory: lane slots issued (32 per entry or per
         // loop trip) by the far loop [0], pass 1 [1] and pass 2 [2] of the pair loop; nodes popped
         // [3], tested lane by lane [4]; leaves [5] and internal nodes [6] opened
-        unsigned *wc = sm.wc[w];
+        unsigned *wc = sm.wc;
         if (lane < 8) wc[lane] = 0u;
-        if (SPH) sm.mum[w][lane] = 0.f;
+        if (SPH) sm.mum[lane] = 0.f;
         if constexpr (DISS) {
-            ds.vs[w][lane] = 0.f;
-            ds.lap[w][lane] = 0.f;
+            sm.vs[lane] = 0.f;
+            sm.lap[lane] = 0.f;
         }
         if constexpr (CHECK) {
-            cks.cs[w][lane] = 0;
-            cks.hs[w][lane] = 0ull;
+            sm.cs[lane] = 0;
+            sm.hs[lane] = 0ull;
         }
         if constexpr (MIXED) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) mx.c[w][k][lane] = 0.f;
+            for (int k = 0; k < 4; ++k) sm.c[k][lane] = 0.f;
         }
         __syncwarp();
 
@@ -294,7 +306,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                 float t, e;
                 two_sum(total, b, t, e);
                 total = t;
-                mx.c[w][k][lane] += e;
+                sm.c[k][lane] += e;
             } else {
                 total += b;
             }
@@ -303,22 +315,23 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         int nfar = 0, nnear = 0;
 
         auto flush_far = [&]() {
+          if constexpr (GRAV) {
             __syncwarp();
             // pad to a whole trip of the loop with empty-mask entries (node 0 is always valid)
             constexpr int TRIP = 2 * EVOL_FAR_UNROLL;
             const int padded = (nfar + TRIP - 1) / TRIP * TRIP;
             if (lane < padded - nfar) {
-                sm.far_id[w][nfar + lane] = 0;
-                sm.far_mask[w][nfar + lane] = 0u;
+                sm.far_id[nfar + lane] = 0;
+                sm.far_mask[nfar + lane] = 0u;
             }
             __syncwarp();
             for (int l = lane; l < padded; l += 32) {
-                const int id = sm.far_id[w][l];
+                const int id = sm.far_id[l];
                 const float4 A = d.nA[id], Q0 = d.nQ0[id], Q1 = d.nQ1[id];
-                float *f = sm.fpair[w][l >> 1] + (l & 1);
+                float *f = sm.fpair[l >> 1] + (l & 1);
                 f[0] = A.x; f[2] = A.y; f[4] = A.z; f[6] = -Q0.w;
                 f[8] = Q0.x; f[10] = Q0.y; f[12] = Q0.z; f[14] = Q1.x; f[16] = Q1.y; f[18] = Q1.z;
-                wfar += __popc(sm.far_mask[w][l]);     // interaction count (this lane's share)
+                wfar += __popc(sm.far_mask[l]);     // interaction count (this lane's share)
             }
             if (lane == 0) wc[0] += 32u * (unsigned)padded;
             __syncwarp();
@@ -334,8 +347,8 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
 #pragma unroll
                 for (int u = 0; u < EVOL_FAR_UNROLL; ++u) {
                     const int pp = (e >> 1) + u;
-                    const uint2 mk = *reinterpret_cast<const uint2 *>(&sm.far_mask[w][2 * pp]);
-                    const ulonglong2 *F = reinterpret_cast<const ulonglong2 *>(sm.fpair[w][pp]);
+                    const uint2 mk = *reinterpret_cast<const uint2 *>(&sm.far_mask[2 * pp]);
+                    const ulonglong2 *F = reinterpret_cast<const ulonglong2 *>(sm.fpair[pp]);
                     const ulonglong2 v0 = F[0], v1 = F[1], v2 = F[2], v3 = F[3], v4 = F[4];
                     // v0 = (x, y), v1 = (z, -M), v2 = (Qxx, Qyy), v3 = (Qzz, Qxy), v4 = (Qxz, Qyz)
                     f32x2 dx = sub2(PX, v0.x), dy = sub2(PY, v0.y), dz = sub2(PZ, v1.x);
@@ -393,42 +406,43 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
             }
             nfar = 0;
             __syncwarp();
+          }
         };
 
         auto flush_near = [&]() {
             __syncwarp();
             // an odd list gets an empty partner entry (no lanes, finite zeros) for the two-wide pass
             if ((nnear & 1) && lane == 0) {
-                sm.near_mask[w][nnear] = 0u;
-                float *f = sm.npair[w][nnear >> 1] + 1;
+                sm.near_mask[nnear] = 0u;
+                float *f = sm.npair[nnear >> 1] + 1;
 #pragma unroll
                 for (int c = 0; c < 6; ++c) f[2 * c] = 0.f;
             }
             for (int l = lane; l < nnear; l += 32) {
-                const int j = sm.near_j[w][l];
-                wpp += __popc(sm.near_mask[w][l]);         // interaction count (this lane's share)
+                const int j = sm.near_j[l];
+                wpp += __popc(sm.near_mask[l]);         // interaction count (this lane's share)
                 const float4 pj = d.pos[j];
                 const float4 gj = d.grav[j];
-                float *f = sm.npair[w][l >> 1] + (l & 1);
+                float *f = sm.npair[l >> 1] + (l & 1);
                 const float te = GRAV ? 2.f / gj.x : 0.f, th = 2.f * gj.z;
                 f[0] = pj.x; f[2] = pj.y; f[4] = pj.z; f[6] = pj.w;
                 f[8] = te * te;
                 f[10] = gj.z > 0.f ? th * th : -1.f;
-                sm.ng[w][l] = gj;
+                sm.ng[l] = gj;
                 if (SPH) {
-                    sm.nh[w][l] = d.hydro[j];
-                    sm.ns[w][l] = d.snd[j];
+                    sm.nh[l] = d.hydro[j];
+                    sm.ns[l] = d.snd[j];
                 }
-                if constexpr (DISS) ds.nd[w][l] = d.diss[j];     // read only for gas pairs
-                if constexpr (CHECK) cks.norig[w][l] = d.orig[j];
+                if constexpr (DISS) sm.nd[l] = d.diss[j];     // read only for gas pairs
+                if constexpr (CHECK) sm.norig[l] = d.orig[j];
             }
             if (lane == 0) wc[1] += 32u * (unsigned)((nnear + 1) & ~1);
             if constexpr (MIXED && GRAV) {
                 // park the running gravity totals; the pair loop sums this flush's block from zero
-                mx.c[w][4][lane] = acc.ax;
-                mx.c[w][5][lane] = acc.ay;
-                mx.c[w][6][lane] = acc.az;
-                mx.c[w][7][lane] = acc.pot;
+                sm.c[4][lane] = acc.ax;
+                sm.c[5][lane] = acc.ay;
+                sm.c[6][lane] = acc.az;
+                sm.c[7][lane] = acc.pot;
                 acc.ax = acc.ay = acc.az = acc.pot = 0.f;
             }
             __syncwarp();
@@ -443,9 +457,10 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                 const f32x2 PX = pk2(pi.x, pi.x), PY = pk2(pi.y, pi.y), PZ = pk2(pi.z, pi.z);
                 f32x2 nax = 0ull, nay = 0ull, naz = 0ull, npot = 0ull;
                 f32x2 ewnxy = 0ull, ewnzw = 0ull;
+#pragma unroll 1               // unrolled, its loads in flight cost a resident block
                 for (int q = 0; q < (nnear + 1) >> 1; ++q) {
-                    const uint2 mk = *reinterpret_cast<const uint2 *>(&sm.near_mask[w][2 * q]);
-                    const ulonglong2 *F = reinterpret_cast<const ulonglong2 *>(sm.npair[w][q]);
+                    const uint2 mk = *reinterpret_cast<const uint2 *>(&sm.near_mask[2 * q]);
+                    const ulonglong2 *F = reinterpret_cast<const ulonglong2 *>(sm.npair[q]);
                     const ulonglong2 v0 = F[0], v1 = F[1], v2 = F[2];   // (x, y), (z, m), (E, H)
                     f32x2 dx = sub2(PX, v0.x), dy = sub2(PY, v0.y), dz = sub2(PZ, v1.x);
                     if (pm) {
@@ -559,7 +574,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                     if (item < nitems) {
                         const int nlo = __popc(olo);
                         const int t = k < nlo ? nth_bit(olo, k) : 32 + nth_bit(ohi, k - nlo);
-                        const float *f = sm.npair[w][t >> 1] + (t & 1);
+                        const float *f = sm.npair[t >> 1] + (t & 1);
                         const float mj = f[6], Ej = f[8], Hj = f[10];
                         const float dx = evol_wrap(po.x - f[0], plen0, pm & 1);
                         const float dy = evol_wrap(po.y - f[2], plen1, pm & 2);
@@ -568,7 +583,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                         // r and 1/r from one reciprocal square root (coincident particles: both 0)
                         const float rinv = r2 > 0.f ? rsqrtf(r2) : 0.f;
                         const float r = r2 * rinv;
-                        const float4 gj = sm.ng[w][t];
+                        const float4 gj = sm.ng[t];
                         if (GRAV && r2 < fmaxf(E_o, Ej)) {              // the same test as pass 1
                             ++wsoft;
                             // symmetrised softened pair force and potential (App. B), each side
@@ -594,21 +609,21 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                         if (SPH && fminf(H_o, Hj) >= 0.f && r2 < fmaxf(H_o, Hj)) {   // as in pass 1
                             ++wsph;
                             if constexpr (CHECK) {
-                                atomicAdd(&cks.cs[w][o], 1);
-                                atomicAdd(&cks.hs[w][o], evol_mix64((unsigned long long)cks.norig[w][t]));
+                                atomicAdd(&sm.cs[o], 1);
+                                atomicAdd(&sm.hs[o], evol_mix64((unsigned long long)sm.norig[t]));
                             }
                             if (kp.wake) {
                                 // wake-up: the owner's step (ticks), recorded at its SPH neighbour
                                 const int jo = d.orig[so];
-                                atomicMin(&d.nbmin[sm.near_j[w][t]], (unsigned)(d.te[jo] - d.tb[jo]));
+                                atomicMin(&d.nbmin[sm.near_j[t]], (unsigned)(d.te[jo] - d.tb[jo]));
                             }
                             if (r2 > 0.f) {
                                 const float4 gi = go;
                                 const float4 hi = d.hydro[so];
                                 const float4 si = d.snd[so];
                                 const float4 di = DISS ? d.diss[so] : z4;
-                                const float4 hj = sm.nh[w][t];
-                                const float4 sj = sm.ns[w][t];
+                                const float4 hj = sm.nh[t];
+                                const float4 sj = sm.ns[t];
                                 const float ihi = si.z, ihj = sj.z;
                                 const float uhi = r * ihi, uhj = r * ihj;
                                 const float iuhi = rinv * gi.z, iuhj = rinv * gj.z;     // h / r
@@ -625,15 +640,15 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                                 float4 dj = z4;
                                 float wij = 0.f, vsig = 0.f;
                                 if constexpr (DISS) {
-                                    dj = ds.nd[w][t];
+                                    dj = sm.nd[t];
                                     wij = vr * rinv;
                                     vsig = si.x + sj.x - fminf(wij, 0.f);
-                                    atomicMax(reinterpret_cast<int *>(&ds.vs[w][o]), __float_as_int(vsig));
+                                    atomicMax(reinterpret_cast<int *>(&sm.vs[o]), __float_as_int(vsig));
                                 }
                                 if (vr < 0.f) {
                                     const float hb = 0.5f * (gi.z + gj.z);
                                     const float mu = hb * vr * rcp_fast(r2 + 0.01f * hb * hb);
-                                    atomicMax(reinterpret_cast<int *>(&sm.mum[w][o]), __float_as_int(-mu));   // |mu|
+                                    atomicMax(reinterpret_cast<int *>(&sm.mum[o]), __float_as_int(-mu));   // |mu|
                                     const float cb = 0.5f * (si.x + sj.x);
                                     const float rb = 0.5f * (si.y + sj.y);
                                     if constexpr (!DISS) {
@@ -708,23 +723,23 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                         acc.hy += tot_[5];
                         acc.hz += tot_[6];
                         acc.du += tot_[7];
-                        if constexpr (DISS) ds.lap[w][lane] += tot_[8];
+                        if constexpr (DISS) sm.lap[lane] += tot_[8];
                     }
                 }
             }
             if constexpr (MIXED && GRAV) {
                 // the block's sums into the parked totals, compensated
                 float b = acc.ax;
-                acc.ax = mx.c[w][4][lane];
+                acc.ax = sm.c[4][lane];
                 add_to(acc.ax, 0, b);
                 b = acc.ay;
-                acc.ay = mx.c[w][5][lane];
+                acc.ay = sm.c[5][lane];
                 add_to(acc.ay, 1, b);
                 b = acc.az;
-                acc.az = mx.c[w][6][lane];
+                acc.az = sm.c[6][lane];
                 add_to(acc.az, 2, b);
                 b = acc.pot;
-                acc.pot = mx.c[w][7][lane];
+                acc.pot = sm.c[7][lane];
                 add_to(acc.pot, 3, b);
             }
             nnear = 0;
@@ -756,9 +771,9 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         // the group bounds live in shared memory for the traversal (read as broadcasts), which keeps
         // them out of the registers the pair loops need
         if (lane == 0) {
-            sm.gbox[w][0] = make_float4(0.5f * (gx0 + gx1), 0.5f * (gy0 + gy1), 0.5f * (gz0 + gz1), 0.f);
-            sm.gbox[w][1] = make_float4(0.5f * (gx1 - gx0), 0.5f * (gy1 - gy0), 0.5f * (gz1 - gz0), 0.f);
-            sm.gbox[w][2] = make_float4(emax, emin, hmax, hmin);
+            sm.gbox[0] = make_float4(0.5f * (gx0 + gx1), 0.5f * (gy0 + gy1), 0.5f * (gz0 + gz1), 0.f);
+            sm.gbox[1] = make_float4(0.5f * (gx1 - gx0), 0.5f * (gy1 - gy0), 0.5f * (gz1 - gz0), 0.f);
+            sm.gbox[2] = make_float4(emax, emin, hmax, hmin);
         }
         __syncwarp();
 
@@ -792,8 +807,8 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         __syncwarp();
         // a traversal pops every node at most once; a larger count can only come from a corrupt
         // tree: stop, flag it and report where
-        long long pops = 0;
-        const long long pop_cap = 2ll * (long long)(*d.nnodes) + 64;
+        unsigned pops = 0u;
+        const unsigned pop_cap = 2u * (unsigned)(*d.nnodes) + 64u;
         while (top > 0 || apos < aend) {
             if (++pops > pop_cap) {
                 if (lane == 0) {
@@ -836,7 +851,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                 const float4 B = d.nB[node];
                 const float4 C = d.nC[node];
                 const float4 A = GRAV ? d.nA[node] : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 G0 = sm.gbox[w][0], G1 = sm.gbox[w][1], G2 = sm.gbox[w][2];
+                const float4 G0 = sm.gbox[0], G1 = sm.gbox[1], G2 = sm.gbox[2];
                 const float gcx = G0.x, gcy = G0.y, gcz = G0.z, gwx = G1.x, gwy = G1.y, gwz = G1.z;
                 const float emax = G2.x, emin = G2.y, hmax = G2.z, hmin = G2.w;
                 const float dx = fabsf(evol_wrap(B.x - gcx, plen0, pm & 1));
@@ -879,9 +894,9 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                 } else {
                     cls = 3;
                 }
-                sm.bA[w][lane] = A;
-                sm.bB[w][lane] = B;
-                sm.bC[w][lane] = C;
+                if constexpr (GRAV) sm.bA[lane] = A;
+                sm.bB[lane] = B;
+                sm.bC[lane] = C;
             }
             __syncwarp();
             // mixed nodes: every lane in the mask applies its own test
@@ -896,8 +911,8 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                 const unsigned Mk = __shfl_sync(0xffffffffu, M, kk);
                 bool far = false;
                 if ((Mk >> lane) & 1u) {
-                    const float4 B = sm.bB[w][kk];
-                    const float4 C = sm.bC[w][kk];
+                    const float4 B = sm.bB[kk];
+                    const float4 C = sm.bC[kk];
                     const float qx = fabsf(evol_wrap(pi.x - B.x, plen0, pm & 1));
                     const float qy = fabsf(evol_wrap(pi.y - B.y, plen1, pm & 2));
                     const float qz = fabsf(evol_wrap(pi.z - B.z, plen2, pm & 4));
@@ -906,11 +921,14 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                     float R = GRAV ? fmaxf(two_eps_i, C.w) : 0.f;
                     if (SPH && gas_i && B.w >= 0.f) R = fmaxf(R, fmaxf(two_h_i, B.w));
                     far = bd2 > R * R;
-                    if (GRAV && far) {
-                        const float4 A = sm.bA[w][kk];
-                        const float dx = evol_wrap(pi.x - A.x, plen0, pmg & 1), dy = evol_wrap(pi.y - A.y, plen1, pmg & 2),
-                                    dz = evol_wrap(pi.z - A.z, plen2, pmg & 4);
-                        far = dx * dx + dy * dy + dz * dz > A.w;
+                    if constexpr (GRAV) {
+                        if (far) {
+                            const float4 A = sm.bA[kk];
+                            const float dx = evol_wrap(pi.x - A.x, plen0, pmg & 1),
+                                        dy = evol_wrap(pi.y - A.y, plen1, pmg & 2),
+                                        dz = evol_wrap(pi.z - A.z, plen2, pmg & 4);
+                            far = dx * dx + dy * dy + dz * dz > A.w;
+                        }
                     }
                 }
                 const unsigned Af = __ballot_sync(0xffffffffu, far);
@@ -934,15 +952,17 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                     }
                 }
             }
-            if (GRAV && fa) {
-                const int cnt = __popc(fa);
-                if (nfar + cnt > FARCAP - 2 * EVOL_FAR_UNROLL + 1) flush_far();
-                if (Ak) {
-                    const int pos = nfar + __popc(fa & ltmask);
-                    sm.far_id[w][pos] = node;
-                    sm.far_mask[w][pos] = Ak;
+            if constexpr (GRAV) {
+                if (fa) {
+                    const int cnt = __popc(fa);
+                    if (nfar + cnt > FARCAP - 2 * EVOL_FAR_UNROLL + 1) flush_far();
+                    if (Ak) {
+                        const int pos = nfar + __popc(fa & ltmask);
+                        sm.far_id[pos] = node;
+                        sm.far_mask[pos] = Ak;
+                    }
+                    nfar += cnt;
                 }
-                nfar += cnt;
             }
             if (pre) continue;               // nothing opened
             // opened leaves: their particles go to the near list
@@ -972,20 +992,20 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                         if (lane < kc) {
                             // the particle itself never pairs with itself: its lane leaves the mask
                             const int j = b + lane, sl = j - g * 32;
-                            sm.near_j[w][nnear + lane] = j;
-                            sm.near_mask[w][nnear + lane] = ok & ~((sl >= 0 && sl < 32) ? (1u << sl) : 0u);
+                            sm.near_j[nnear + lane] = j;
+                            sm.near_mask[nnear + lane] = ok & ~((sl >= 0 && sl < 32) ? (1u << sl) : 0u);
                         }
                     } else {
                         // active list: the group's lanes hold arbitrary sorted positions; the lane
                         // whose particle is entry b + q marks slot q, and that bit leaves the mask
-                        if (lane < kc) sm.gself[w][lane] = 0u;
+                        if (lane < kc) sm.gself[lane] = 0u;
                         __syncwarp();
-                        const int mine = sm.gs[w][lane];
-                        if (mine >= b && mine < b + kc) sm.gself[w][mine - b] = 1u << lane;
+                        const int mine = sm.gs[lane];
+                        if (mine >= b && mine < b + kc) sm.gself[mine - b] = 1u << lane;
                         __syncwarp();
                         if (lane < kc) {
-                            sm.near_j[w][nnear + lane] = b + lane;
-                            sm.near_mask[w][nnear + lane] = ok & ~sm.gself[w][lane];
+                            sm.near_j[nnear + lane] = b + lane;
+                            sm.near_mask[nnear + lane] = ok & ~sm.gself[lane];
                         }
                         __syncwarp();
                     }
@@ -1030,8 +1050,8 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         double thx = acc.hx, thy = acc.hy, thz = acc.hz, tdu = acc.du;
         if constexpr (MIXED) {
             // total = running sum + compensation, in FP64
-            tax += (double)mx.c[w][0][lane]; tay += (double)mx.c[w][1][lane];
-            taz += (double)mx.c[w][2][lane]; tpot += (double)mx.c[w][3][lane];
+            tax += (double)sm.c[0][lane]; tay += (double)sm.c[1][lane];
+            taz += (double)sm.c[2][lane]; tpot += (double)sm.c[3][lane];
         }
         if (valid) {
             float ax = 0.f, ay = 0.f, az = 0.f, pot = 0.f;
@@ -1051,7 +1071,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
             d.acc[s] = make_float4(ax, ay, az, pot);
             if (SPH) {
                 d.dudt[s] = gas_i ? (float)tdu : 0.f;
-                d.mumax[s] = gas_i ? sm.mum[w][lane] : 0.f;
+                d.mumax[s] = gas_i ? sm.mum[lane] : 0.f;
                 const float4 hv = d.hydro[s];
                 d.vah[s] = gas_i ? (float)(hv.x * thx + hv.y * thy + hv.z * thz) : 0.f;
             }
@@ -1061,8 +1081,8 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                     // alpha_tau h_i / v^sig_i; the switches of alpha (Eq. alphaswitch) and alpha^u
                     const float4 sn = d.snd[s], di = d.diss[s];
                     const float h_i = g0.z;
-                    const float vs = fmaxf(ds.vs[w][lane], 2.f * sn.x);
-                    const float lap = ds.lap[w][lane];
+                    const float vs = fmaxf(sm.vs[lane], 2.f * sn.x);
+                    const float lap = sm.lap[lane];
                     const float itau = vs / (kp.alpha_tau * h_i);
                     d.vsig[s] = vs;
                     d.lapu[s] = lap;
@@ -1078,10 +1098,10 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
             if constexpr (CHECK) {
                 d.hash3[3 * s + 0] = hfar;
                 d.hash3[3 * s + 1] = hnear;
-                d.hash3[3 * s + 2] = cks.hs[w][lane];
+                d.hash3[3 * s + 2] = sm.hs[lane];
                 d.cnt3[3 * s + 0] = cfar;
                 d.cnt3[3 * s + 1] = cpp;
-                d.cnt3[3 * s + 2] = cks.cs[w][lane];
+                d.cnt3[3 * s + 2] = sm.cs[lane];
             }
         }
         // interaction counters, per lane: summed over the warp
