@@ -309,9 +309,12 @@ __device__ __forceinline__ unsigned long long evol_mix64(unsigned long long z)
     return z ^ (z >> 31);
 }
 
-__device__ __forceinline__ float evol_wrap(float d, float len, int periodic)
+// Nearest image on an axis of length len (il = 1/len, 0 for an axis that is not periodic): the nearest
+// integer by adding and subtracting 1.5 2^23, exact below 2^22 box lengths.
+__device__ __forceinline__ float evol_nearest(float d, float len, float il)
 {
-    return periodic ? d - len * rintf(d / len) : d;
+    const float k = (d * il + 12582912.f) - 12582912.f;
+    return d - len * k;
 }
 
 // ---- force-walk super-groups: groups of 32 list entries per super-group, list capacities -----

@@ -108,18 +108,10 @@ struct LenSmem {
     int cj[FLOW ? CC : 1];            // sorted index of each candidate
 };
 
-// Nearest image on an axis of length len (il = 1/len, 0 for an axis that is not periodic): rounding to
-// the nearest integer by adding and subtracting 1.5 2^23, exact below 2^22 box lengths.
-__device__ __forceinline__ float wrap_m(float d, float len, float il)
-{
-    const float k = (d * il + 12582912.f) - 12582912.f;
-    return d - len * k;
-}
-
 template <bool PER>
 __device__ __forceinline__ float image(float d, const evol_kparams &kp, int a)
 {
-    return PER ? wrap_m(d, kp.plen[a], kp.pinv[a]) : d;
+    return PER ? evol_nearest(d, kp.plen[a], kp.pinv[a]) : d;
 }
 
 // Minimum and maximum over the warp's lanes (one reduction instruction each).

@@ -243,12 +243,11 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
     const int nlist = kp.active ? d.acts[n] : n;
     const int ngroups = (nlist + 31) >> 5;
     // periodic axes: SPH alone, or gravity in a periodic cube (EWALD: nearest images plus the
-    // tabulated correction of the replicas, Sect. 4.3); pmg: the periodic axes of the gravity tests
-    const int pm = ((SPH && !GRAV) || EWALD) ? kp.periodic_mask : 0;
-    const int pmg = EWALD ? kp.periodic_mask : 0;
+    // tabulated correction of the replicas, Sect. 4.3)
+    constexpr bool PER = (SPH && !GRAV) || EWALD;
     const float iL = EWALD ? 1.f / kp.ewald_L : 0.f;
     const float side0 = EWALD ? d.fcube[3] : 0.f;     // root cube side (periodic gravity: one system)
-    const float plen0 = kp.plen[0], plen1 = kp.plen[1], plen2 = kp.plen[2];
+    auto nearest = [&](float x, int a) -> float { return PER ? evol_nearest(x, kp.plen[a], kp.pinv[a]) : x; };
     const float inv_pi = 1.f / EVOL_PI_F;
 
     for (;;) {
@@ -355,9 +354,9 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                     if constexpr (EWALD) {
                         // nearest image of the centre of mass, and the node's replicas beyond it
                         // (monopole: its mass at the centre of mass)
-                        dx = pk2(evol_wrap(lo2(dx), plen0, pmg & 1), evol_wrap(hi2(dx), plen0, pmg & 1));
-                        dy = pk2(evol_wrap(lo2(dy), plen1, pmg & 2), evol_wrap(hi2(dy), plen1, pmg & 2));
-                        dz = pk2(evol_wrap(lo2(dz), plen2, pmg & 4), evol_wrap(hi2(dz), plen2, pmg & 4));
+                        dx = pk2(nearest(lo2(dx), 0), nearest(hi2(dx), 0));
+                        dy = pk2(nearest(lo2(dy), 1), nearest(hi2(dy), 1));
+                        dz = pk2(nearest(lo2(dz), 2), nearest(hi2(dz), 2));
                         if ((mk.x >> lane) & 1u) {
                             const float ex = lo2(dx), ey = lo2(dy), ez = lo2(dz);
                             const Ew2 c = ewald_lookup2(kp.ewald_tab, ex, ey, ez, kp.ewald_sc);
@@ -463,10 +462,10 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                     const ulonglong2 *F = reinterpret_cast<const ulonglong2 *>(sm.npair[q]);
                     const ulonglong2 v0 = F[0], v1 = F[1], v2 = F[2];   // (x, y), (z, m), (E, H)
                     f32x2 dx = sub2(PX, v0.x), dy = sub2(PY, v0.y), dz = sub2(PZ, v1.x);
-                    if (pm) {
-                        dx = pk2(evol_wrap(lo2(dx), plen0, pm & 1), evol_wrap(hi2(dx), plen0, pm & 1));
-                        dy = pk2(evol_wrap(lo2(dy), plen1, pm & 2), evol_wrap(hi2(dy), plen1, pm & 2));
-                        dz = pk2(evol_wrap(lo2(dz), plen2, pm & 4), evol_wrap(hi2(dz), plen2, pm & 4));
+                    if (PER && kp.periodic_mask) {
+                        dx = pk2(nearest(lo2(dx), 0), nearest(hi2(dx), 0));
+                        dy = pk2(nearest(lo2(dy), 1), nearest(hi2(dy), 1));
+                        dz = pk2(nearest(lo2(dz), 2), nearest(hi2(dz), 2));
                     }
                     const f32x2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
                     const float ra = lo2(r2), rb = hi2(r2);
@@ -576,9 +575,9 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                         const int t = k < nlo ? nth_bit(olo, k) : 32 + nth_bit(ohi, k - nlo);
                         const float *f = sm.npair[t >> 1] + (t & 1);
                         const float mj = f[6], Ej = f[8], Hj = f[10];
-                        const float dx = evol_wrap(po.x - f[0], plen0, pm & 1);
-                        const float dy = evol_wrap(po.y - f[2], plen1, pm & 2);
-                        const float dz = evol_wrap(po.z - f[4], plen2, pm & 4);
+                        const float dx = nearest(po.x - f[0], 0);
+                        const float dy = nearest(po.y - f[2], 1);
+                        const float dz = nearest(po.z - f[4], 2);
                         const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));     // as in pass 1
                         // r and 1/r from one reciprocal square root (coincident particles: both 0)
                         const float rinv = r2 > 0.f ? rsqrtf(r2) : 0.f;
@@ -854,9 +853,9 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                 const float4 G0 = sm.gbox[0], G1 = sm.gbox[1], G2 = sm.gbox[2];
                 const float gcx = G0.x, gcy = G0.y, gcz = G0.z, gwx = G1.x, gwy = G1.y, gwz = G1.z;
                 const float emax = G2.x, emin = G2.y, hmax = G2.z, hmin = G2.w;
-                const float dx = fabsf(evol_wrap(B.x - gcx, plen0, pm & 1));
-                const float dy = fabsf(evol_wrap(B.y - gcy, plen1, pm & 2));
-                const float dz = fabsf(evol_wrap(B.z - gcz, plen2, pm & 4));
+                const float dx = fabsf(nearest(B.x - gcx, 0));
+                const float dy = fabsf(nearest(B.y - gcy, 1));
+                const float dz = fabsf(nearest(B.z - gcz, 2));
                 // nearest and farthest distance of a group point from the node box
                 const float nx = fmaxf(dx - (C.x + gwx), 0.f), ny = fmaxf(dy - (C.y + gwy), 0.f),
                             nz = fmaxf(dz - (C.z + gwz), 0.f);
@@ -878,8 +877,8 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                     open_all = true;
                 }
                 if (GRAV) {
-                    const float ax = fabsf(evol_wrap(A.x - gcx, plen0, pmg & 1)), ay = fabsf(evol_wrap(A.y - gcy, plen1, pmg & 2)),
-                                az = fabsf(evol_wrap(A.z - gcz, plen2, pmg & 4));
+                    const float ax = fabsf(nearest(A.x - gcx, 0)), ay = fabsf(nearest(A.y - gcy, 1)),
+                                az = fabsf(nearest(A.z - gcz, 2));
                     const float mx = fmaxf(ax - gwx, 0.f), my = fmaxf(ay - gwy, 0.f), mz = fmaxf(az - gwz, 0.f);
                     const float Mx = ax + gwx, My = ay + gwy, Mz = az + gwz;
                     acc_all = acc_all && (mx * mx + my * my + mz * mz > A.w * (1.f + TAU));
@@ -913,9 +912,9 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                 if ((Mk >> lane) & 1u) {
                     const float4 B = sm.bB[kk];
                     const float4 C = sm.bC[kk];
-                    const float qx = fabsf(evol_wrap(pi.x - B.x, plen0, pm & 1));
-                    const float qy = fabsf(evol_wrap(pi.y - B.y, plen1, pm & 2));
-                    const float qz = fabsf(evol_wrap(pi.z - B.z, plen2, pm & 4));
+                    const float qx = fabsf(nearest(pi.x - B.x, 0));
+                    const float qy = fabsf(nearest(pi.y - B.y, 1));
+                    const float qz = fabsf(nearest(pi.z - B.z, 2));
                     const float ex = fmaxf(qx - C.x, 0.f), ey = fmaxf(qy - C.y, 0.f), ez = fmaxf(qz - C.z, 0.f);
                     const float bd2 = ex * ex + ey * ey + ez * ez;
                     float R = GRAV ? fmaxf(two_eps_i, C.w) : 0.f;
@@ -924,9 +923,9 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
                     if constexpr (GRAV) {
                         if (far) {
                             const float4 A = sm.bA[kk];
-                            const float dx = evol_wrap(pi.x - A.x, plen0, pmg & 1),
-                                        dy = evol_wrap(pi.y - A.y, plen1, pmg & 2),
-                                        dz = evol_wrap(pi.z - A.z, plen2, pmg & 4);
+                            const float dx = nearest(pi.x - A.x, 0),
+                                        dy = nearest(pi.y - A.y, 1),
+                                        dz = nearest(pi.z - A.z, 2);
                             far = dx * dx + dy * dy + dz * dz > A.w;
                         }
                     }
@@ -1138,9 +1137,8 @@ __global__ void __launch_bounds__(32, 24) k_super(evol_dev d, evol_kparams kp, i
     const int lane = threadIdx.x;
     const int n = kp.n;
     const int nlist = kp.active ? d.acts[n] : n;
-    const int pm = ((SPH && !GRAV) || EWALD) ? kp.periodic_mask : 0;
-    const int pmg = EWALD ? kp.periodic_mask : 0;
-    const float plen0 = kp.plen[0], plen1 = kp.plen[1], plen2 = kp.plen[2];
+    constexpr bool PER = (SPH && !GRAV) || EWALD;
+    auto nearest = [&](float x, int a) -> float { return PER ? evol_nearest(x, kp.plen[a], kp.pinv[a]) : x; };
     const float side0 = EWALD ? d.fcube[3] : 0.f;
     int *stk = reinterpret_cast<int *>(d.wstack + (size_t)blockIdx.x * kp.stack_stride);
     const int stack_cap = 2 * kp.stack_cap;
@@ -1223,9 +1221,9 @@ __global__ void __launch_bounds__(32, 24) k_super(evol_dev d, evol_kparams kp, i
                     const float4 B = d.nB[node];
                     const float4 C = d.nC[node];
                     const float4 A = GRAV ? d.nA[node] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float dx = fabsf(evol_wrap(B.x - gcx, plen0, pm & 1));
-                    const float dy = fabsf(evol_wrap(B.y - gcy, plen1, pm & 2));
-                    const float dz = fabsf(evol_wrap(B.z - gcz, plen2, pm & 4));
+                    const float dx = fabsf(nearest(B.x - gcx, 0));
+                    const float dy = fabsf(nearest(B.y - gcy, 1));
+                    const float dz = fabsf(nearest(B.z - gcz, 2));
                     const float nx = fmaxf(dx - (C.x + gwx), 0.f), ny = fmaxf(dy - (C.y + gwy), 0.f),
                                 nz = fmaxf(dz - (C.z + gwz), 0.f);
                     const float fx = fmaxf(dx + gwx - C.x, 0.f), fy = fmaxf(dy + gwy - C.y, 0.f),
@@ -1244,8 +1242,8 @@ __global__ void __launch_bounds__(32, 24) k_super(evol_dev d, evol_kparams kp, i
                         open_all = true;
                     }
                     if (GRAV) {
-                        const float ax = fabsf(evol_wrap(A.x - gcx, plen0, pmg & 1)), ay = fabsf(evol_wrap(A.y - gcy, plen1, pmg & 2)),
-                                    az = fabsf(evol_wrap(A.z - gcz, plen2, pmg & 4));
+                        const float ax = fabsf(nearest(A.x - gcx, 0)), ay = fabsf(nearest(A.y - gcy, 1)),
+                                    az = fabsf(nearest(A.z - gcz, 2));
                         const float mx = fmaxf(ax - gwx, 0.f), my = fmaxf(ay - gwy, 0.f), mz = fmaxf(az - gwz, 0.f);
                         const float Mx = ax + gwx, My = ay + gwy, Mz = az + gwz;
                         acc_all = acc_all && (mx * mx + my * my + mz * mz > A.w * (1.f + TAU));
@@ -1383,7 +1381,10 @@ int evol_launch_walk(evol_ctx *c, const evol_particles *p, const evol_params *pr
     kp.adaptive = prm->adaptive_softening;
     kp.use_tc = prm->use_tc_gradient;
     kp.periodic_mask = prm->periodic_mask;
-    for (int a = 0; a < 3; ++a) kp.plen[a] = prm->periodic_hi[a] - prm->periodic_lo[a];
+    for (int a = 0; a < 3; ++a) {
+        kp.plen[a] = prm->periodic_hi[a] - prm->periodic_lo[a];
+        kp.pinv[a] = (prm->periodic_mask >> a) & 1 ? 1.f / kp.plen[a] : 0.f;
+    }
     kp.stack_cap = (int)c->wstack_lim;
     kp.stack_stride = (int)c->wstack_cap;
     kp.active = c->bins_active;
