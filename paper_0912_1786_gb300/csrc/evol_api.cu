@@ -38,7 +38,7 @@ void free_all(evol_ctx *c)
     evol_dev &d = c->d;
     void *ptrs[] = {d.pos, d.vel, d.grav, d.hydro, d.snd, d.vah, d.orig, d.inv, d.divv_h, d.divv_e, d.mumax, d.dt, d.time, d.len_h, d.len_eps, d.nh, d.omega,
                     d.diss, d.curlv_h, d.vsig, d.lapu, d.dalpha, d.dalpha_u, d.tb, d.te, d.bact, d.pred_tau,
-                    d.pers, d.actf, d.acts, d.act, d.gbase, d.glist, d.gpos, d.sg_acc, d.sg_front, d.sg_info, d.sg_rad, d.sg_stat, d.nbmin, d.bt, d.ewald,
+                    d.pers, d.actf, d.acts, d.act, d.gbase, d.glist, d.gpos, d.sg_acc, d.sg_front, d.sg_info, d.sg_rad, d.sg_stat, d.wpart, d.nbmin, d.bt, d.ewald,
                     d.zeta, d.rho, d.neps, d.ups, d.X, d.acc, d.dudt, d.keys_a, d.keys_b, d.vals_a, d.vals_b,
                     d.hist, d.lcp, d.cnt, d.base, d.scan_part, d.nbeg, d.nend, d.nlev, d.nnext, d.nparent,
                     d.nnch, d.narrive, d.nA, d.nB, d.nC, d.nQ0, d.nQ1, d.nM64, d.nC64, d.nQ64, d.nBmin,
@@ -317,6 +317,10 @@ int evol_create(evol_ctx **out, int64_t max_n, void *stream)
         const int64_t nsg = n / (32 * EVOL_SG_GROUPS) + 2;     // super-groups of the force walk
         rc |= dalloc(&d.sg_acc, nsg * EVOL_SG_ACAP); rc |= dalloc(&d.sg_front, nsg * EVOL_SG_FCAP);
         rc |= dalloc(&d.sg_info, nsg); rc |= dalloc(&d.sg_rad, 4 * nsg); rc |= dalloc(&d.sg_stat, 2);
+        // items of the force walk in parts (walk_parts): 16 per group at most, and at most 17/8 per warp of
+        // the grid, which holds 32 per SM or less
+        const int64_t ngr = n / 32 + 1, most = (int64_t)c->num_sms * 32 * 17 / 8;
+        rc |= dalloc(&d.wpart, (16 * ngr < most ? 16 * ngr : most) * EVOL_PART_FLOATS);
     }
     rc |= dalloc(&d.nbmin, n); rc |= dalloc(&d.bt, 8);
     rc |= dalloc(&d.ewald, (int64_t)EVOL_EWALD_M * EVOL_EWALD_M * EVOL_EWALD_M);

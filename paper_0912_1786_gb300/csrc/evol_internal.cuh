@@ -55,6 +55,7 @@ struct evol_dev {
     // their counts (-1: walk from the root)
     int32_t *sg_acc, *sg_front;
     int2 *sg_info;
+    float *wpart;            // force walk, groups in parts: each part's sums (EVOL_PART_FLOATS)
     float *sg_rad;           // length solves: search radius of each quarter of a super-group
     unsigned long long *sg_stat;     // and the candidates of all super-groups, and their number
     unsigned *nbmin;                // sorted: smallest active-neighbour step (wake-up)
@@ -321,6 +322,9 @@ __device__ __forceinline__ float evol_nearest(float d, float len, float il)
 #define EVOL_SG_GROUPS 8
 #define EVOL_SG_ACAP 3072
 #define EVOL_SG_FCAP 768
+// Per part of a group walked in parts, 32 lanes of each: a, phi (without G), a_hyd, du/dt, max |mu|, max
+// v^sig, lap u, and the compensation terms of a and phi.
+#define EVOL_PART_FLOATS 512
 
 // ---- periodic gravity (Ewald, Sect. 4.3) ----------------------------------------------------
 // Correction table for a cube of side 1: (f_x, f_y, f_z, g) at the grid points (i, j, k) / (2 N) of the
@@ -345,6 +349,7 @@ struct evol_kparams {
     // positions, ascending; its length at d.acts[n]); the force walk also records, per SPH
     // neighbour, the smallest step (ticks) of an active particle next to it (wake-up)
     int active, wake;
+    int part_slots;          // force walk in parts: warps of that variant's grid (0: whole groups only)
     int super;               // the force walk's groups start from their super-group's lists
     int lists;               // the length solves' blocks take their leaves from super-group lists
     int lsub;                // particles per warp of the length solves (1..32; 0: from their number)

@@ -37,6 +37,23 @@ constexpr int FARCAP = 64;
 constexpr int NEARCAP = 64;
 constexpr int SG_GROUPS = EVOL_SG_GROUPS;   // groups per super-group (see k_super)
 
+// Parts of a group's walk (PARTS variants).  A set with fewer groups than the grid has warps leaves most of
+// the chip idle while each warp works through its group alone.  There 2^k items share a group: each takes
+// every 2^k-th frontier node of its super-group and a slice of the nodes accepted for all, and leaves its
+// sums in d.wpart; k_walk_finish adds them up.  As many parts as give each warp of the grid about two items,
+// at most 16 (a part pays for the group's bounds and for partly filled batches): 1000 particles 0.25 ms whole
+// -> 0.11 (16 parts; 0.13 with 4, 0.12 with 32), 4096 particles 0.40 -> 0.16, 49,152 particles 1.11 -> 0.91 (2
+// parts; 0.97 with 4, 1.13 with 8).  With more groups than warps whole groups are as fast.
+constexpr int PART_MAX = 4;       // at most 2^4 parts
+
+__device__ __forceinline__ int walk_parts(int ngroups, int slots)
+{
+    if (ngroups > slots) return 0;
+    int k = 0;
+    while (k < PART_MAX && (ngroups << (k + 1)) <= 2 * slots + slots / 8) ++k;
+    return k;
+}
+
 constexpr float TAU = 1e-5f;      // safety margin of the group-level bounds
 
 // One warp's shared memory: one base address for all of it, every array at a constant offset.
@@ -221,16 +238,72 @@ template <>
 struct CheckSmem<false> {
 };
 
+// A particle's sums over the whole walk.
+struct WalkTotals {
+    double ax, ay, az, pot;           // gravity (without G)
+    double hx, hy, hz, du;            // SPH
+    float mu, vs, lap;                // largest |mu|, largest v^sig, Brookshaw lap u
+};
+
+// Results of the particle at sorted position s (mass m, gravity operands g0) from its sums.
+template <bool GRAV, bool SPH, bool DISS, bool EWALD>
+__device__ __forceinline__ void write_particle(const evol_dev &d, const evol_kparams &kp, int s, float m, float4 g0,
+                                               bool gas_i, const WalkTotals &t)
+{
+    float ax = 0.f, ay = 0.f, az = 0.f, pot = 0.f;
+    if (GRAV) {
+        // self term of the potential: m_i phi(0, eps_i) = -7/5 m_i / eps_i
+        const double G = kp.G;
+        ax = (float)(G * t.ax);
+        ay = (float)(G * t.ay);
+        az = (float)(G * t.az);
+        double self_img = 0.0;
+        if (EWALD) self_img = (double)m * (double)kp.ewald_tab[0].w * (double)(1.f / kp.ewald_L);   // own replicas
+        pot = (float)(G * (t.pot - 1.4 * (double)m * (double)g0.x + self_img));
+    }
+    ax += (float)t.hx;
+    ay += (float)t.hy;
+    az += (float)t.hz;
+    d.acc[s] = make_float4(ax, ay, az, pot);
+    if (SPH) {
+        d.dudt[s] = gas_i ? (float)t.du : 0.f;
+        d.mumax[s] = gas_i ? t.mu : 0.f;
+        const float4 hv = d.hydro[s];
+        d.vah[s] = gas_i ? (float)(hv.x * t.hx + hv.y * t.hy + hv.z * t.hz) : 0.f;
+    }
+    if constexpr (DISS) {
+        if (gas_i) {
+            // v^sig_i = max(2 c_i, max_j v^sig_ij) (the self pair has w = 0); tau_i =
+            // alpha_tau h_i / v^sig_i; the switches of alpha (Eq. alphaswitch) and alpha^u
+            const float4 sn = d.snd[s], di = d.diss[s];
+            const float h_i = g0.z;
+            const float vs = fmaxf(t.vs, 2.f * sn.x);
+            const float lap = t.lap;
+            const float itau = vs / (kp.alpha_tau * h_i);
+            d.vsig[s] = vs;
+            d.lapu[s] = lap;
+            if (kp.var_alpha)
+                d.dalpha[s] = -(di.x - kp.alpha_min) * itau + kp.alpha_source * di.y * fmaxf(0.f, -d.divv_h[s]);
+            if (kp.conduction) {
+                const float src = kp.cond_source == EVOL_COND_SRC_LINEAR ? 0.1f * h_i * fabsf(lap)
+                                                                         : h_i * fabsf(lap) * rsqrtf(di.z);
+                d.dalpha_u[s] = -(di.w - kp.alpha_u_min) * itau + src;
+            }
+        }
+    }
+}
+
 // Register budgets, chosen so that no variant spills to local memory: the gravity + SPH walk (the
 // production form, plain or mixed) fits five blocks per SM (at most 102 registers), the SPH-only walk, which
 // holds no far list, six (80); the walks with the dissipation variants (DISS), the plain gravity-only walk
 // and the plain gravity-only periodic one (EWALD) four (128 registers); the other periodic and mixed DISS
-// walks three; the check-mode variants one.  What made room: one base address for all of a warp's shared
+// walks three; the check-mode variants one; the PARTS variants, for sets that do not fill the chip, three or
+// four.  What made room: one base address for all of a warp's shared
 // memory, and a first pair pass that is not unrolled (gravity only, 2^20 Plummer particles: three blocks and
 // 6.7 ms before, four and 5.9 ms now; SPH only, 1.05 M-particle shock tube: five blocks and 3.6 ms before,
 // six and 2.8 ms now).
-template <bool GRAV, bool SPH, bool MIXED, bool CHECK, bool DISS, bool EWALD>
-__global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIXED) ? 4 : (EWALD || (MIXED && DISS)) ? 3 : DISS || !SPH ? 4 : !GRAV ? 6 : EVOL_WALK_MINB) k_walk(evol_dev d, evol_kparams kp, unsigned long long *queue)
+template <bool GRAV, bool SPH, bool MIXED, bool CHECK, bool DISS, bool EWALD, bool PARTS>
+__global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : PARTS ? (GRAV && SPH || MIXED && DISS ? 3 : 4) : (EWALD && !SPH && !MIXED) ? 4 : (EWALD || (MIXED && DISS)) ? 3 : DISS || !SPH ? 4 : !GRAV ? 6 : EVOL_WALK_MINB) k_walk(evol_dev d, evol_kparams kp, unsigned long long *queue)
 {
     struct WarpSmem : WalkSmem, FarSmem<GRAV>, DissSmem<DISS>, CheckSmem<CHECK>, MixSmem<MIXED> {
     };
@@ -242,9 +315,14 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
     // individual time steps: groups of 32 consecutive entries of the active list
     const int nlist = kp.active ? d.acts[n] : n;
     const int ngroups = (nlist + 31) >> 5;
+    // 2^psh items per group; of the PARTS variant and the one with whole groups, the one that the number of
+    // groups asks for does the work
+    const int psh = kp.part_slots ? walk_parts(ngroups, kp.part_slots) : 0;
+    if ((psh > 0) != PARTS) return;
     // periodic axes: SPH alone, or gravity in a periodic cube (EWALD: nearest images plus the
     // tabulated correction of the replicas, Sect. 4.3)
     constexpr bool PER = (SPH && !GRAV) || EWALD;
+    constexpr int FAR_UNROLL = EWALD ? 2 : EVOL_FAR_UNROLL;   // the table lookups bound the periodic loop
     const float iL = EWALD ? 1.f / kp.ewald_L : 0.f;
     const float side0 = EWALD ? d.fcube[3] : 0.f;     // root cube side (periodic gravity: one system)
     auto nearest = [&](float x, int a) -> float { return PER ? evol_nearest(x, kp.plen[a], kp.pinv[a]) : x; };
@@ -254,7 +332,13 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         int g = 0;
         if (lane == 0) g = (int)atomicAdd(queue, 1ull);
         g = __shfl_sync(0xffffffffu, g, 0);
-        if (g >= ngroups) break;
+        if constexpr (PARTS) {
+            if (g >= ngroups << psh) break;
+            if (lane == 0) sm.wc[7] = (unsigned)g;       // the item: group << psh | part
+            g >>= psh;
+        } else {
+            if (g >= ngroups) break;
+        }
         const int e = g * 32 + lane;
         const bool valid = e < nlist;
         const int s = kp.active ? (valid ? d.act[e] : 0) : e;
@@ -266,7 +350,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         const float4 g0 = valid ? d.grav[s] : make_float4(0.f, 0.f, 0.f, 0.f);
         const bool gas_i = SPH && valid && g0.z > 0.f;
         const bool active = valid && (GRAV || gas_i);
-        const float ie_i = g0.x, two_eps_i = GRAV && active ? 2.f / g0.x : 0.f;
+        const float two_eps_i = GRAV && active ? 2.f / g0.x : 0.f;
         const float two_h_i = gas_i ? 2.f * g0.z : 0.f;
         // squared near radii of the pair tests: softened gravity inside max(E_i, E_j), SPH inside
         // max(H_i, H_j) when both are gas (H = -1 marks a particle that is not)
@@ -282,7 +366,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         // loop trip) by the far loop [0], pass 1 [1] and pass 2 [2] of the pair loop; nodes popped
         // [3], tested lane by lane [4]; leaves [5] and internal nodes [6] opened
         unsigned *wc = sm.wc;
-        if (lane < 8) wc[lane] = 0u;
+        if (lane < 7) wc[lane] = 0u;
         if (SPH) sm.mum[lane] = 0.f;
         if constexpr (DISS) {
             sm.vs[lane] = 0.f;
@@ -317,7 +401,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
           if constexpr (GRAV) {
             __syncwarp();
             // pad to a whole trip of the loop with empty-mask entries (node 0 is always valid)
-            constexpr int TRIP = 2 * EVOL_FAR_UNROLL;
+            constexpr int TRIP = 2 * FAR_UNROLL;
             const int padded = (nfar + TRIP - 1) / TRIP * TRIP;
             if (lane < padded - nfar) {
                 sm.far_id[nfar + lane] = 0;
@@ -344,7 +428,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
             f32x2 ewxy = 0ull, ewzw = 0ull;                             // Ewald corrections (x M)
             for (int e = 0; e < padded; e += TRIP) {
 #pragma unroll
-                for (int u = 0; u < EVOL_FAR_UNROLL; ++u) {
+                for (int u = 0; u < FAR_UNROLL; ++u) {
                     const int pp = (e >> 1) + u;
                     const uint2 mk = *reinterpret_cast<const uint2 *>(&sm.far_mask[2 * pp]);
                     const ulonglong2 *F = reinterpret_cast<const ulonglong2 *>(sm.fpair[pp]);
@@ -789,12 +873,18 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
             // the stack, the nodes it accepted for all as batches that skip the node tests (they
             // count only as far nodes, and as accepted nodes in check mode)
             const size_t sgb = (size_t)(g / SG_GROUPS);
-            for (int k = lane; k < sgi.y; k += 32)
-                stk[k] = make_int2(d.sg_front[sgb * EVOL_SG_FCAP + k], (int)rootmask);
-            top = sgi.y;
+            const int part = PARTS ? (int)(wc[7] & ((1u << psh) - 1u)) : 0;
+            top = PARTS ? (sgi.y - part + (1 << psh) - 1) >> psh : sgi.y;
+            for (int k = lane; k < top; k += 32)
+                stk[k] = make_int2(d.sg_front[sgb * EVOL_SG_FCAP + (PARTS ? (k << psh) + part : k)], (int)rootmask);
             alist = d.sg_acc + sgb * EVOL_SG_ACAP;
             aend = (GRAV || CHECK) ? sgi.x : 0;
-        } else {
+            if constexpr (PARTS) {
+                apos = (aend * part) >> psh;
+                aend = (aend * (part + 1)) >> psh;
+            }
+        } else if (!PARTS || (wc[7] & ((1u << psh) - 1u)) == 0u) {
+            // (without lists the first part walks alone)
             // one stack entry per system present in the group: its root with the mask of its lanes
             const int myroot = active ? d.sys_root[d.sys_sorted[s]] : -1;
             const unsigned peers = __match_any_sync(0xffffffffu, myroot);
@@ -954,7 +1044,7 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
             if constexpr (GRAV) {
                 if (fa) {
                     const int cnt = __popc(fa);
-                    if (nfar + cnt > FARCAP - 2 * EVOL_FAR_UNROLL + 1) flush_far();
+                    if (nfar + cnt > FARCAP - 2 * FAR_UNROLL + 1) flush_far();
                     if (Ak) {
                         const int pos = nfar + __popc(fa & ltmask);
                         sm.far_id[pos] = node;
@@ -1045,55 +1135,40 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
         if (GRAV && nfar) flush_far();
         if (nnear) flush_near();
 
-        double tax = acc.ax, tay = acc.ay, taz = acc.az, tpot = acc.pot;
-        double thx = acc.hx, thy = acc.hy, thz = acc.hz, tdu = acc.du;
-        if constexpr (MIXED) {
-            // total = running sum + compensation, in FP64
-            tax += (double)sm.c[0][lane]; tay += (double)sm.c[1][lane];
-            taz += (double)sm.c[2][lane]; tpot += (double)sm.c[3][lane];
-        }
-        if (valid) {
-            float ax = 0.f, ay = 0.f, az = 0.f, pot = 0.f;
+        if constexpr (PARTS) {
+            // this part's sums, for k_walk_finish
+            float *mine = d.wpart + (size_t)wc[7] * EVOL_PART_FLOATS + lane;
             if (GRAV) {
-                // self term of the potential: m_i phi(0, eps_i) = -7/5 m_i / eps_i
-                const double G = kp.G;
-                ax = (float)(G * tax);
-                ay = (float)(G * tay);
-                az = (float)(G * taz);
-                double self_img = 0.0;
-                if (EWALD) self_img = (double)pi.w * (double)kp.ewald_tab[0].w * (double)iL;   // own replicas
-                pot = (float)(G * (tpot - 1.4 * (double)pi.w * (double)ie_i + self_img));
+                mine[0] = acc.ax; mine[32] = acc.ay; mine[64] = acc.az; mine[96] = acc.pot;
             }
-            ax += (float)thx;
-            ay += (float)thy;
-            az += (float)thz;
-            d.acc[s] = make_float4(ax, ay, az, pot);
             if (SPH) {
-                d.dudt[s] = gas_i ? (float)tdu : 0.f;
-                d.mumax[s] = gas_i ? sm.mum[lane] : 0.f;
-                const float4 hv = d.hydro[s];
-                d.vah[s] = gas_i ? (float)(hv.x * thx + hv.y * thy + hv.z * thz) : 0.f;
+                mine[128] = acc.hx; mine[160] = acc.hy; mine[192] = acc.hz; mine[224] = acc.du;
+                mine[256] = sm.mum[lane];
             }
             if constexpr (DISS) {
-                if (gas_i) {
-                    // v^sig_i = max(2 c_i, max_j v^sig_ij) (the self pair has w = 0); tau_i =
-                    // alpha_tau h_i / v^sig_i; the switches of alpha (Eq. alphaswitch) and alpha^u
-                    const float4 sn = d.snd[s], di = d.diss[s];
-                    const float h_i = g0.z;
-                    const float vs = fmaxf(sm.vs[lane], 2.f * sn.x);
-                    const float lap = sm.lap[lane];
-                    const float itau = vs / (kp.alpha_tau * h_i);
-                    d.vsig[s] = vs;
-                    d.lapu[s] = lap;
-                    if (kp.var_alpha)
-                        d.dalpha[s] = -(di.x - kp.alpha_min) * itau + kp.alpha_source * di.y * fmaxf(0.f, -d.divv_h[s]);
-                    if (kp.conduction) {
-                        const float src = kp.cond_source == EVOL_COND_SRC_LINEAR ? 0.1f * h_i * fabsf(lap)
-                                                                                 : h_i * fabsf(lap) * rsqrtf(di.z);
-                        d.dalpha_u[s] = -(di.w - kp.alpha_u_min) * itau + src;
-                    }
-                }
+                mine[288] = sm.vs[lane];
+                mine[320] = sm.lap[lane];
             }
+            if constexpr (MIXED) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) mine[352 + 32 * k] = sm.c[k][lane];
+            }
+        } else if (valid) {
+            WalkTotals t;
+            t.ax = acc.ax; t.ay = acc.ay; t.az = acc.az; t.pot = acc.pot;
+            t.hx = acc.hx; t.hy = acc.hy; t.hz = acc.hz; t.du = acc.du;
+            if constexpr (MIXED) {
+                // total = running sum + compensation, in FP64
+                t.ax += (double)sm.c[0][lane]; t.ay += (double)sm.c[1][lane];
+                t.az += (double)sm.c[2][lane]; t.pot += (double)sm.c[3][lane];
+            }
+            t.mu = SPH ? sm.mum[lane] : 0.f;
+            t.vs = t.lap = 0.f;
+            if constexpr (DISS) {
+                t.vs = sm.vs[lane];
+                t.lap = sm.lap[lane];
+            }
+            write_particle<GRAV, SPH, DISS, EWALD>(d, kp, s, pi.w, g0, gas_i, t);
             if constexpr (CHECK) {
                 d.hash3[3 * s + 0] = hfar;
                 d.hash3[3 * s + 1] = hnear;
@@ -1120,6 +1195,41 @@ __global__ void __launch_bounds__(WK_THREADS, CHECK ? 1 : (EWALD && !SPH && !MIX
             for (int q = 0; q < 7; ++q) atomicAdd(&d.counters[9 + q], (unsigned long long)wc[q]);
         }
     }
+}
+
+// The results of groups walked in parts: each particle's sums over the parts, added up in their order and in
+// FP64.
+template <bool GRAV, bool SPH, bool MIXED, bool DISS>
+__global__ void __launch_bounds__(WK_THREADS) k_walk_finish(evol_dev d, evol_kparams kp)
+{
+    const int nlist = kp.active ? d.acts[kp.n] : kp.n;
+    const int psh = walk_parts((nlist + 31) >> 5, kp.part_slots);
+    const int e = blockIdx.x * WK_THREADS + threadIdx.x;
+    if (psh == 0 || e >= nlist) return;
+    const int s = kp.active ? d.act[e] : e;
+    const float4 g0 = d.grav[s];
+    const bool gas_i = SPH && g0.z > 0.f;
+    WalkTotals t = {0., 0., 0., 0., 0., 0., 0., 0., 0.f, 0.f, 0.f};
+    const float *all = d.wpart + ((size_t)(e >> 5) << psh) * EVOL_PART_FLOATS + (e & 31);
+#pragma unroll 4
+    for (int p = 0; p < 1 << psh; ++p) {
+        const float *q = all + p * EVOL_PART_FLOATS;
+        if (GRAV) {
+            t.ax += q[0]; t.ay += q[32]; t.az += q[64]; t.pot += q[96];
+        }
+        if (SPH) {
+            t.hx += q[128]; t.hy += q[160]; t.hz += q[192]; t.du += q[224];
+            t.mu = fmaxf(t.mu, q[256]);
+        }
+        if constexpr (DISS) {
+            t.vs = fmaxf(t.vs, q[288]);
+            t.lap += q[320];
+        }
+        if constexpr (MIXED) {
+            t.ax += q[352]; t.ay += q[384]; t.az += q[416]; t.pot += q[448];
+        }
+    }
+    write_particle<GRAV, SPH, DISS, false>(d, kp, s, d.pos[s].w, g0, gas_i, t);
 }
 
 // Super-groups: 8 consecutive groups (256 consecutive entries of the particle list) walk the top of
@@ -1312,19 +1422,36 @@ __global__ void __launch_bounds__(32, 24) k_super(evol_dev d, evol_kparams kp, i
     }
 }
 
-template <bool GRAV, bool SPH, bool MIXED, bool CHECK, bool DISS, bool EWALD>
-void launch_walk(evol_ctx *c, const evol_kparams &kp)
+template <bool GRAV, bool SPH, bool MIXED, bool CHECK, bool DISS, bool EWALD, bool PARTS>
+int walk_grid(evol_ctx *c)
 {
     static int blocks_per_sm = -1;
     if (blocks_per_sm < 0) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_walk<GRAV, SPH, MIXED, CHECK, DISS, EWALD>,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_walk<GRAV, SPH, MIXED, CHECK, DISS, EWALD, PARTS>,
                                                       WK_THREADS, 0);
         if (blocks_per_sm < 1) blocks_per_sm = 1;
         if (blocks_per_sm > 8) blocks_per_sm = 8;          // stack slots exist for 32 warps per SM
     }
+    return c->num_sms * blocks_per_sm;
+}
+
+template <bool GRAV, bool SPH, bool MIXED, bool CHECK, bool DISS, bool EWALD>
+void launch_walk(evol_ctx *c, evol_kparams kp)
+{
     unsigned long long *q = c->d.counters + 4;
     cudaMemsetAsync(q, 0, sizeof(unsigned long long), c->stream);
-    k_walk<GRAV, SPH, MIXED, CHECK, DISS, EWALD><<<c->num_sms * blocks_per_sm, WK_THREADS, 0, c->stream>>>(c->d, kp, q);
+    if constexpr (!EWALD && !CHECK) {
+        // in parts where the groups do not fill the grid (of an active list, whose length only the device
+        // knows, both variants are launched and one returns)
+        const int grid = walk_grid<GRAV, SPH, MIXED, CHECK, DISS, EWALD, true>(c);
+        if (kp.active || (kp.n + 31) / 32 <= grid * WK_WARPS) {
+            kp.part_slots = grid * WK_WARPS;
+            k_walk<GRAV, SPH, MIXED, CHECK, DISS, EWALD, true><<<grid, WK_THREADS, 0, c->stream>>>(c->d, kp, q);
+            k_walk_finish<GRAV, SPH, MIXED, DISS><<<(kp.n + WK_THREADS - 1) / WK_THREADS, WK_THREADS, 0, c->stream>>>(c->d, kp);
+        }
+    }
+    k_walk<GRAV, SPH, MIXED, CHECK, DISS, EWALD, false>
+        <<<walk_grid<GRAV, SPH, MIXED, CHECK, DISS, EWALD, false>(c), WK_THREADS, 0, c->stream>>>(c->d, kp, q);
 }
 
 template <bool GRAV, bool SPH, bool DISS, bool EWALD>
