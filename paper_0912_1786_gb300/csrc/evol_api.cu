@@ -292,7 +292,7 @@ int evol_create(evol_ctx **out, int64_t max_n, void *stream)
     c->device = dev;
     c->num_sms = prop.multiProcessorCount;
     c->stream = (cudaStream_t)stream;
-    c->sort_blocks = (max_n + 4095) / 4096;
+    c->sort_blocks = (max_n + 2047) / 2048;
     c->bbox_blocks = c->num_sms * 2;
     c->diag_blocks = c->num_sms * 2;
     c->wstack_slots = (int64_t)c->num_sms * 32;      // the walk and length grids use at most 32 warps per SM
@@ -327,7 +327,12 @@ int evol_create(evol_ctx **out, int64_t max_n, void *stream)
     if (!rc && cudaMallocHost((void **)&c->h_bt, 8 * sizeof(unsigned long long)) != cudaSuccess) rc = EVOL_ENOMEM;
     rc |= dalloc(&d.dt, 4); rc |= dalloc(&d.time, 1);
     rc |= dalloc(&d.keys_a, n); rc |= dalloc(&d.keys_b, n); rc |= dalloc(&d.vals_a, n); rc |= dalloc(&d.vals_b, n);
-    rc |= dalloc(&d.hist, 256 * c->sort_blocks + 1);
+    {
+        // one pass's counts, or 11 passes' (8 digits and three of the system id) of a set with fused passes
+        const int64_t tiles = max_n < EVOL_SORT_FUSED_MAX ? c->sort_blocks : EVOL_SORT_FUSED_MAX / 2048;
+        const int64_t one = 256 * c->sort_blocks + 1, all = 11 * 256 * tiles;
+        rc |= dalloc(&d.hist, one > all ? one : all);
+    }
     rc |= dalloc(&d.lcp, n); rc |= dalloc(&d.cnt, n + 1); rc |= dalloc(&d.base, n + 1);
     rc |= dalloc(&d.scan_part, scan_parts);
     rc |= dalloc(&d.nbeg, nn); rc |= dalloc(&d.nend, nn); rc |= dalloc(&d.nlev, nn); rc |= dalloc(&d.nnext, nn);

@@ -10,6 +10,7 @@
 #define EVOL_MAXLEVEL 21          // 21 bits per axis, 63-bit Morton keys
 #define EVOL_WARP 32
 #define EVOL_NCOUNTERS 32
+#define EVOL_SORT_FUSED_MAX 131072   // largest set whose radix passes are one kernel each (see tree.cu)
 #define EVOL_PI_F 3.14159265358979f
 
 // ---- device error word: first error wins ------------------------------------------------
@@ -67,7 +68,7 @@ struct evol_dev {
     // sort
     uint64_t *keys_a, *keys_b;
     int32_t *vals_a, *vals_b;
-    uint32_t *hist;          // 256 * nblocks
+    uint32_t *hist;          // digit counts of the sort's tiles (of every pass where passes are fused)
     // tree construction
     int8_t *lcp;             // d_i: common octal digits of keys i-1, i (-1: i starts a system)
     int32_t *cnt, *base;     // nodes beginning at each sorted position, and its exclusive scan
@@ -108,7 +109,7 @@ struct evol_ctx {
     int device, num_sms;
     cudaStream_t stream;
     evol_dev d;
-    int64_t sort_blocks;
+    int64_t sort_blocks;     // tiles of the radix sort
     int64_t bbox_blocks;
     int64_t wstack_slots, wstack_cap;
     int64_t wstack_lim;      // entries the walks may use per warp (<= wstack_cap)

@@ -162,16 +162,16 @@ __global__ void k_diag_partial(int n, int n_gas, int have_sph, evol_dev d, doubl
     }
 }
 
+// A warp per quantity (one thread going through the 304 partial sums took 27 us).
 __global__ void k_diag_final(int nparts, const double *part, const int32_t *nnodes,
                              const unsigned long long *counters, double *diag)
 {
-    int k = threadIdx.x;
-    if (k < DG_N) {
-        double x = 0.0;
-        for (int b = 0; b < nparts; ++b) x += part[b * DG_N + k];
-        diag[k] = x;
-    }
-    if (k == 0) {
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double x = 0.0;
+    for (int b = lane; b < nparts; b += 32) x += part[b * DG_N + k];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane == 0) diag[k] = x;
+    if (threadIdx.x == 0) {
         diag[11] = (double)*nnodes;
         diag[12] = (double)counters[0];
         diag[13] = (double)counters[1];
@@ -585,7 +585,7 @@ int evol_launch_diagnostics(evol_ctx *c, const evol_particles *p, const evol_par
 {
     int nb = (int)c->diag_blocks;
     k_diag_partial<<<nb, DG_THREADS, 0, c->stream>>>((int)p->n, (int)p->n_gas, prm->sph, c->d, c->d.diag_part);
-    k_diag_final<<<1, 32, 0, c->stream>>>(nb, c->d.diag_part, c->d.nnodes, c->d.counters, c->d.diag);
+    k_diag_final<<<1, 32 * DG_N, 0, c->stream>>>(nb, c->d.diag_part, c->d.nnodes, c->d.counters, c->d.diag);
     return evol_cuda_ok(cudaGetLastError());
 }
 

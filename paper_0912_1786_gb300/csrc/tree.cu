@@ -20,11 +20,19 @@ namespace {
 
 constexpr int BB_THREADS = 256;
 constexpr int RS_THREADS = 256;
-constexpr int RS_ITEMS = 16;
+constexpr int RS_ITEMS = 8;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
 constexpr int SC_THREADS = 1024;
 constexpr int SC_ITEMS = 4;
 constexpr int SC_TILE = SC_THREADS * SC_ITEMS;
+// The sort's three forms, by size; whole tree builds of a Plummer sphere on one GB300, ms.  Up to RANK_MAX
+// each key's position is counted directly, n^2 comparisons in one launch (against fused passes: 4095
+// particles 0.146 / 0.196, 8191 0.181 / 0.223, 12000 0.205 / 0.237, 24000 0.275 / 0.241).  Up to FUSED_MAX a
+// radix pass is one kernel whose blocks each sum every tile's digit counts, a cost that grows as n^2 (against
+// histogram, scan and scatter: 16384 0.237 / 0.258, 131072 0.311 / 0.340, 200000 0.371 / 0.343).
+constexpr int RANK_MAX = 12288;
+constexpr int FUSED_MAX = EVOL_SORT_FUSED_MAX;
+constexpr int SCAN_ONE_MAX = 4 * SC_TILE;    // scans up to this size by one block
 
 // ---------------------------------------------------------------------------------------
 // Root cube
@@ -64,19 +72,38 @@ __global__ void k_bbox_partial(int n, const float *__restrict__ x, const float *
     }
 }
 
-// corner = per-axis minimum; side = smallest power of two >= extent * (1 + 2^-20) (1 if 0)
-__global__ void k_bbox_final(int nparts, const float *__restrict__ part, double *cube, float *fcube)
+// Minimum (components 0..2) and maximum (3..5) of six values over a block of at most 32 warps; the result
+// is on thread 0.
+__device__ __forceinline__ void block_bounds(float v[6])
 {
-    if (threadIdx.x != 0) return;
-    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int b = 0; b < nparts; ++b)
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = fminf(lo[a], part[b * 6 + a]);
-            hi[a] = fmaxf(hi[a], part[b * 6 + 3 + a]);
+    __shared__ float sh[32][6];
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int a = 0; a < 6; ++a)
+        for (int o = 16; o > 0; o >>= 1) {
+            const float t = __shfl_xor_sync(0xffffffffu, v[a], o);
+            v[a] = a < 3 ? fminf(v[a], t) : fmaxf(v[a], t);
         }
+    if (l == 0)
+        for (int a = 0; a < 6; ++a) sh[w][a] = v[a];
+    __syncthreads();
+    if (w == 0)
+#pragma unroll
+        for (int a = 0; a < 6; ++a) {
+            v[a] = l < nw ? sh[l][a] : (a < 3 ? INFINITY : -INFINITY);
+            for (int o = 16; o > 0; o >>= 1) {
+                const float t = __shfl_xor_sync(0xffffffffu, v[a], o);
+                v[a] = a < 3 ? fminf(v[a], t) : fmaxf(v[a], t);
+            }
+        }
+}
+
+// corner = per-axis minimum; side = smallest power of two >= extent * (1 + 2^-20) (1 if 0)
+__device__ __forceinline__ void write_cube(const float v[6], double *cube, float *fcube)
+{
     double ext = 0.0;
     for (int a = 0; a < 3; ++a) {
-        double e = (double)hi[a] - (double)lo[a];
+        double e = (double)v[3 + a] - (double)v[a];
         ext = e > ext ? e : ext;
     }
     double target = ext * (1.0 + ldexp(1.0, -20));
@@ -87,11 +114,30 @@ __global__ void k_bbox_final(int nparts, const float *__restrict__ part, double 
         s = (fr == 0.5) ? ldexp(1.0, ex - 1) : ldexp(1.0, ex);
     }
     for (int a = 0; a < 3; ++a) {
-        cube[a] = (double)lo[a];
-        fcube[a] = lo[a];
+        cube[a] = (double)v[a];
+        fcube[a] = v[a];
     }
     cube[3] = s;
     fcube[3] = (float)s;
+}
+
+// One system's cube from the partial bounds, a block wide (one thread going through the 304 partials took
+// 28 us), and its offsets.
+__global__ void k_bbox_final(int n, int nparts, const float *__restrict__ part, double *cube, float *fcube,
+                             int32_t *sys_off)
+{
+    float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    for (int b = threadIdx.x; b < nparts; b += blockDim.x)
+        for (int a = 0; a < 3; ++a) {
+            v[a] = fminf(v[a], part[b * 6 + a]);
+            v[3 + a] = fmaxf(v[3 + a], part[b * 6 + 3 + a]);
+        }
+    block_bounds(v);
+    if (threadIdx.x == 0) {
+        write_cube(v, cube, fcube);
+        sys_off[0] = 0;
+        sys_off[1] = n;
+    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -118,8 +164,10 @@ __device__ __forceinline__ double key_scale(double side)
     return ldexp(1.0, EVOL_MAXLEVEL + 1 - e);
 }
 
+// hist, if given, counts the first digit of the radix sort per tile (zeroed by the caller).
 __global__ void k_keys(int n, const float *__restrict__ x, const float *__restrict__ y, const float *__restrict__ z,
-                       const double *__restrict__ cube, uint64_t *__restrict__ keys, int32_t *__restrict__ vals)
+                       const double *__restrict__ cube, uint64_t *__restrict__ keys, int32_t *__restrict__ vals,
+                       int32_t *__restrict__ hist)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -133,8 +181,21 @@ __global__ void k_keys(int n, const float *__restrict__ x, const float *__restri
         s = s > 2097151.0 ? 2097151.0 : s;
         q[a] = (uint64_t)s;
     }
-    keys[i] = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
+    const uint64_t key = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
+    keys[i] = key;
     vals[i] = i;
+    if (hist) atomicAdd(&hist[(i / RS_TILE) * 256 + (int)(key & 255u)], 1);
+}
+
+__device__ __forceinline__ int sys_of_pos(const int32_t *__restrict__ sys_off, int nsys, int s)
+{
+    // largest k with sys_off[k] <= s
+    int lo = 0, hi = nsys;           // sys_off[0] = 0 <= s < sys_off[nsys]
+    while (hi - lo > 1) {
+        int mid = (lo + hi) >> 1;
+        if (sys_off[mid] <= s) lo = mid; else hi = mid;
+    }
+    return lo;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -221,6 +282,88 @@ __global__ void k_scan_down(int n, const int32_t *in, int32_t *out, const int32_
     if (write_total && blockIdx.x == 0 && threadIdx.x == 0) out[n] = part[nparts];
 }
 
+// A whole scan by one block.
+__global__ void __launch_bounds__(SC_THREADS) k_scan_one(int n, const int32_t *in, int32_t *out, int write_total)
+{
+    __shared__ int32_t sh[32];
+    int32_t carry = 0;
+    for (int b = 0; b < n; b += SC_TILE) {
+        const int base = b + threadIdx.x * SC_ITEMS;
+        int32_t v[SC_ITEMS], s = 0, tot;
+#pragma unroll
+        for (int k = 0; k < SC_ITEMS; ++k) {
+            v[k] = base + k < n ? in[base + k] : 0;
+            s += v[k];
+        }
+        int32_t pre = carry + block_excl_scan(s, sh, tot);
+#pragma unroll
+        for (int k = 0; k < SC_ITEMS; ++k) {
+            if (base + k < n) out[base + k] = pre;
+            pre += v[k];
+        }
+        carry += tot;
+    }
+    if (write_total && threadIdx.x == 0) out[n] = carry;
+}
+
+// ---------------------------------------------------------------------------------------
+// Small sets: the sorted position of key i is the number of keys before it in (key, index) order, counted
+// directly.  A block ranks 32 keys, one per lane, its eight warps going through eighths of every tile of
+// keys; bound by its integer comparisons (1000 particles 5.4 us; 40 launches of a radix sort before).  Several systems: keys of the same system only, from its offset.
+// ---------------------------------------------------------------------------------------
+template <bool SYS>
+__global__ void __launch_bounds__(256) k_rank_sort(int n, const uint64_t *__restrict__ keys,
+                                                   const int32_t *__restrict__ sys_off, int nsys,
+                                                   uint64_t *__restrict__ kout, int32_t *__restrict__ vout)
+{
+    constexpr int TILE = 1024;
+    __shared__ __align__(16) uint64_t tile[TILE];
+    __shared__ int32_t cnt[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * 32, i = i0 + lane;
+    const uint64_t key = i < n ? keys[i] : 0ull;
+    // this key's system: [b, e)
+    int b = 0, e = n;
+    if (SYS && i < n) {
+        const int sy = sys_of_pos(sys_off, nsys, i);
+        b = sys_off[sy];
+        e = sys_off[sy + 1];
+    }
+    int c = 0;
+    for (int t0 = 0; t0 < n; t0 += TILE) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < TILE; t += 256) tile[t] = t0 + t < n ? keys[t0 + t] : ~0ull;
+        __syncthreads();
+        const int j0 = t0 + w * (TILE / 8);
+        if (SYS || (j0 < i0 + 32 && j0 + TILE / 8 > i0)) {
+#pragma unroll 4
+            for (int t = 0; t < TILE / 8; ++t) {
+                const int j = j0 + t;
+                const bool before = tile[w * (TILE / 8) + t] < key + (j < i ? 1u : 0u);   // ties by index
+                c += before && (!SYS || (j >= b && j < e)) ? 1 : 0;
+            }
+        } else {
+            const uint64_t lim = key + (j0 < i0 ? 1u : 0u);
+            const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(tile + w * (TILE / 8));
+#pragma unroll 8
+            for (int t = 0; t < TILE / 16; ++t) {
+                const ulonglong2 k2 = p[t];
+                c += k2.x < lim ? 1 : 0;
+                c += k2.y < lim ? 1 : 0;
+            }
+        }
+    }
+    cnt[w][lane] = c;
+    __syncthreads();
+    if (w == 0 && i < n) {
+        int pos = b;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) pos += cnt[q][lane];
+        kout[pos] = key;
+        vout[pos] = i;
+    }
+}
+
 // ---------------------------------------------------------------------------------------
 // Stable LSD radix sort, 8-bit digits, 64-bit keys with int32 values.
 // ---------------------------------------------------------------------------------------
@@ -239,53 +382,87 @@ __global__ void k_rs_hist(int n, const uint64_t *__restrict__ keys, int shift, i
     hist[threadIdx.x * nblocks + blockIdx.x] = (int32_t)h[threadIdx.x];
 }
 
+// One pass's scatter of a tile.  A warp owns 32 RS_ITEMS consecutive keys and ranks them 32 at a time (the
+// lanes with its digit before it, and the warp's count of that digit so far); the warps' counts are then
+// turned into positions.  FUSED: offs holds every tile's histogram, from which the block sums its own
+// offsets (at most FUSED_MAX / RS_TILE loads a thread), and the next digit's histogram is counted as the keys
+// are written (next), so that a pass is one kernel; else offs is the scanned histogram, digit by digit.
+template <bool FUSED>
 __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(int n, const uint64_t *__restrict__ kin,
                                                            const int32_t *__restrict__ vin, uint64_t *__restrict__ kout,
                                                            int32_t *__restrict__ vout, int shift,
-                                                           const int32_t *__restrict__ offs, int nblocks)
+                                                           const int32_t *__restrict__ offs, int nblocks,
+                                                           int32_t *__restrict__ next)
 {
     constexpr int NW = RS_THREADS / 32;
     __shared__ uint32_t wcnt[NW][256];
-    __shared__ uint32_t run[256];
-    __shared__ uint32_t goff[256];
-    int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    goff[t] = (uint32_t)offs[t * nblocks + blockIdx.x];
-    run[t] = 0;
-    unsigned lt = (1u << lane) - 1u;
-    int base = blockIdx.x * RS_TILE;
+    __shared__ int32_t sh[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+#pragma unroll
+    for (int k = 0; k < NW; ++k) wcnt[k][t] = 0;
+    __syncthreads();
+    const unsigned lt = (1u << lane) - 1u;
+    const int base = blockIdx.x * RS_TILE + w * (32 * RS_ITEMS) + lane;
+    uint64_t key[RS_ITEMS];
+    uint32_t rank[RS_ITEMS];
+#pragma unroll
+    for (int r = 0; r < RS_ITEMS; ++r) key[r] = base + 32 * r < n ? kin[base + 32 * r] : 0ull;
+#pragma unroll
     for (int r = 0; r < RS_ITEMS; ++r) {
-#pragma unroll
-        for (int k = 0; k < NW; ++k) wcnt[k][t] = 0;
-        __syncthreads();
-        int i = base + r * RS_THREADS + t;
-        bool valid = i < n;
-        uint64_t key = valid ? kin[i] : 0ull;
-        int32_t val = valid ? vin[i] : 0;
-        unsigned d = valid ? ((unsigned)(key >> shift) & 255u) : 256u;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        unsigned rank = __popc(peers & lt);
-        if (valid && (__ffs(peers) - 1) == lane) wcnt[w][d] = __popc(peers);
-        __syncthreads();
-        uint32_t acc = run[t];
-#pragma unroll
-        for (int k = 0; k < NW; ++k) {
-            uint32_t c = wcnt[k][t];
-            wcnt[k][t] = acc;
-            acc += c;
+        const unsigned d = base + 32 * r < n ? ((unsigned)(key[r] >> shift) & 255u) : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const int leader = __ffs(peers) - 1;
+        uint32_t before = 0;
+        if (lane == leader && d < 256u) {
+            before = wcnt[w][d];
+            wcnt[w][d] = before + __popc(peers);
         }
-        run[t] = acc;
-        __syncthreads();
-        if (valid) {
-            uint32_t pos = goff[d] + wcnt[w][d] + rank;
-            kout[pos] = key;
-            vout[pos] = val;
+        rank[r] = __shfl_sync(0xffffffffu, before, leader) + __popc(peers & lt);
+        __syncwarp();
+    }
+    // digit t: where this tile's keys go
+    uint32_t run;
+    if (FUSED) {
+        int32_t mine = 0, all = 0, tot;
+#pragma unroll 8
+        for (int q = 0; q < nblocks; ++q) {
+            const int32_t c = offs[q * 256 + t];
+            all += c;
+            mine += q < (int)blockIdx.x ? c : 0;
         }
+        run = (uint32_t)(block_excl_scan(all, sh, tot) + mine);
+    } else {
+        run = (uint32_t)offs[t * nblocks + blockIdx.x];
         __syncthreads();
     }
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        const uint32_t c = wcnt[k][t];
+        wcnt[k][t] = run;
+        run += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RS_ITEMS; ++r)
+        if (base + 32 * r < n) {
+            const uint32_t pos = wcnt[w][(unsigned)(key[r] >> shift) & 255u] + rank[r];
+            kout[pos] = key[r];
+            vout[pos] = vin[base + 32 * r];
+            if (FUSED && next) atomicAdd(&next[(pos / RS_TILE) * 256 + ((unsigned)(key[r] >> (shift + 8)) & 255u)], 1);
+        }
+}
+
+// d_i = common leading octal digits of keys i-1 and i; -1 where i starts a system (a forest of
+// independent trees, one per system, in one pre-order list).
+__device__ __forceinline__ int8_t lcp_of(const uint64_t *__restrict__ keys, int i, bool starts)
+{
+    if (starts) return -1;
+    const uint64_t x = keys[i - 1] ^ keys[i];
+    return x == 0 ? (int8_t)EVOL_MAXLEVEL : (int8_t)((__clzll((long long)x) - 1) / 3);
 }
 
 // ---------------------------------------------------------------------------------------
-// Permutation into sorted order.
+// Permutation into sorted order, and each position's system and common digits with its predecessor.
 // ---------------------------------------------------------------------------------------
 __global__ void k_permute(int n, int n_gas, const int32_t *__restrict__ perm, const float *__restrict__ x,
                           const float *__restrict__ y, const float *__restrict__ z, const float *__restrict__ vx,
@@ -294,11 +471,16 @@ __global__ void k_permute(int n, int n_gas, const int32_t *__restrict__ perm, co
                           float4 *__restrict__ pos, float4 *__restrict__ vel, float *__restrict__ lh,
                           float *__restrict__ le, int32_t *__restrict__ orig, int32_t *__restrict__ inv,
                           const float *__restrict__ pred_dt, const float *__restrict__ pred_acc, int64_t stride,
-                          const float *__restrict__ pred_tau)
+                          const float *__restrict__ pred_tau, const uint64_t *__restrict__ keys,
+                          const int32_t *__restrict__ sys_off, int nsys, int8_t *__restrict__ lcp,
+                          int32_t *__restrict__ sys_sorted)
 {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     int j = perm[s];
+    const int sy = nsys > 1 ? sys_of_pos(sys_off, nsys, s) : 0;
+    sys_sorted[s] = sy;
+    lcp[s] = lcp_of(keys, s, s == (nsys > 1 ? sys_off[sy] : 0));
     bool gas = j < n_gas;
     pos[s] = make_float4(x[j], y[j], z[j], m[j]);
     float4 v = make_float4(vx ? vx[j] : 0.f, vy ? vy[j] : 0.f, vz ? vz[j] : 0.f, (gas && u) ? u[j] : 0.f);
@@ -324,34 +506,6 @@ __global__ void k_permute(int n, int n_gas, const int32_t *__restrict__ perm, co
 // ---------------------------------------------------------------------------------------
 // Node construction.
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ int sys_of_pos(const int32_t *__restrict__ sys_off, int nsys, int s)
-{
-    // largest k with sys_off[k] <= s
-    int lo = 0, hi = nsys;           // sys_off[0] = 0 <= s < sys_off[nsys]
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (sys_off[mid] <= s) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-// d_i = common leading octal digits of keys i-1 and i; -1 where i starts a system (a forest of
-// independent trees, one per system, in one pre-order list).
-__global__ void k_lcp(int n, const uint64_t *__restrict__ keys, const int32_t *__restrict__ sys_off, int nsys,
-                      int8_t *__restrict__ lcp, int32_t *__restrict__ sys_sorted)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int sy = sys_of_pos(sys_off, nsys, i);
-    sys_sorted[i] = sy;
-    if (i == sys_off[sy]) {
-        lcp[i] = -1;
-        return;
-    }
-    uint64_t x = keys[i - 1] ^ keys[i];
-    lcp[i] = x == 0 ? (int8_t)EVOL_MAXLEVEL : (int8_t)((__clzll((long long)x) - 1) / 3);
-}
-
 // Does the level-lam run containing position i hold more than `leaf` particles?
 __device__ __forceinline__ bool run_exceeds(int n, const int8_t *__restrict__ lcp, int i, int lam, int leaf)
 {
@@ -440,9 +594,12 @@ __global__ void k_link(const int32_t *__restrict__ nnodes, int leaf, const int32
                        const int32_t *__restrict__ nend, const int32_t *__restrict__ nlev,
                        const int32_t *__restrict__ nnext, int32_t *__restrict__ nparent, int32_t *__restrict__ nnch,
                        int32_t *__restrict__ narrive, int4 *__restrict__ nI, int4 *__restrict__ nK0,
-                       int4 *__restrict__ nK1)
+                       int4 *__restrict__ nK1, int nsys, const int32_t *__restrict__ sys_off,
+                       const int32_t *__restrict__ base, int32_t *__restrict__ sys_root)
 {
     int nn = *nnodes;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nsys; k += gridDim.x * blockDim.x)
+        sys_root[k] = base[sys_off[k]];
     for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nn; id += gridDim.x * blockDim.x) {
         narrive[id] = 0;
         if (nlev[id] == 0) nparent[id] = -1;     // the root of a system
@@ -747,68 +904,33 @@ __global__ void k_node_lengths(const int32_t *__restrict__ nnodes, int n_gas, co
 }
 
 // ---- several independent systems (batched): per-system cube and keys ----------------------
-__global__ void k_set_single(int n, int32_t *sys_off)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        sys_off[0] = 0;
-        sys_off[1] = n;
-    }
-}
-
 // one block per system: its cube from its own particles
-__global__ void k_bbox_sys(const int32_t *__restrict__ sys_off, const float *__restrict__ x,
+// (also one small system: offsets 0, n are then written here, n > 0)
+__global__ void k_bbox_sys(int n, int32_t *__restrict__ sys_off, const float *__restrict__ x,
                            const float *__restrict__ y, const float *__restrict__ z, double *cube, float *fcube,
                            int *err)
 {
     const int k = blockIdx.x;
-    const int b = sys_off[k], e = sys_off[k + 1];
-    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    const int b = n > 0 ? 0 : sys_off[k], e = n > 0 ? n : sys_off[k + 1];
+    float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    bool bad = false;
+#pragma unroll 4
     for (int i = b + threadIdx.x; i < e; i += blockDim.x) {
-        float v[3] = {x[i], y[i], z[i]};
-        if (!(isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]))) evol_flag(err, EVOL_ENAN);
+        const float p[3] = {x[i], y[i], z[i]};
+        bad |= !(isfinite(p[0]) && isfinite(p[1]) && isfinite(p[2]));
         for (int a = 0; a < 3; ++a) {
-            lo[a] = fminf(lo[a], v[a]);
-            hi[a] = fmaxf(hi[a], v[a]);
+            v[a] = fminf(v[a], p[a]);
+            v[3 + a] = fmaxf(v[3 + a], p[a]);
         }
     }
-    for (int a = 0; a < 3; ++a)
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-            hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-        }
-    __shared__ float sred[BB_THREADS / 32][6];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0)
-        for (int a = 0; a < 3; ++a) {
-            sred[w][a] = lo[a];
-            sred[w][3 + a] = hi[a];
-        }
-    __syncthreads();
+    if (bad) evol_flag(err, EVOL_ENAN);
+    block_bounds(v);
     if (threadIdx.x == 0) {
-        double ext = 0.0;
-        float L[3], H[3];
-        for (int a = 0; a < 3; ++a) {
-            L[a] = sred[0][a];
-            H[a] = sred[0][3 + a];
-            for (int q = 1; q < BB_THREADS / 32; ++q) {
-                L[a] = fminf(L[a], sred[q][a]);
-                H[a] = fmaxf(H[a], sred[q][3 + a]);
-            }
-            double ee = (double)H[a] - (double)L[a];
-            ext = ee > ext ? ee : ext;
+        write_cube(v, cube + 4 * k, fcube + 4 * k);
+        if (n > 0) {
+            sys_off[0] = 0;
+            sys_off[1] = n;
         }
-        double target = ext * (1.0 + ldexp(1.0, -20)), side = 1.0;
-        if (target > 0.0) {
-            int ex;
-            double fr = frexp(target, &ex);
-            side = (fr == 0.5) ? ldexp(1.0, ex - 1) : ldexp(1.0, ex);
-        }
-        for (int a = 0; a < 3; ++a) {
-            cube[4 * k + a] = (double)L[a];
-            fcube[4 * k + a] = L[a];
-        }
-        cube[4 * k + 3] = side;
-        fcube[4 * k + 3] = (float)side;
     }
 }
 
@@ -829,22 +951,27 @@ __device__ __forceinline__ uint64_t key_of(float x, float y, float z, const doub
 // keys in the caller's order, each relative to its own system's cube
 __global__ void k_keys_sys(int n, const float *__restrict__ x, const float *__restrict__ y,
                            const float *__restrict__ z, const int32_t *__restrict__ sys_off, int nsys,
-                           const double *__restrict__ cube, uint64_t *__restrict__ keys, int32_t *__restrict__ vals)
+                           const double *__restrict__ cube, uint64_t *__restrict__ keys, int32_t *__restrict__ vals,
+                           int32_t *__restrict__ hist)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int sy = sys_of_pos(sys_off, nsys, i);
-    keys[i] = key_of(x[i], y[i], z[i], cube + 4 * sy);
+    const uint64_t key = key_of(x[i], y[i], z[i], cube + 4 * sy);
+    keys[i] = key;
     vals[i] = i;
+    if (hist) atomicAdd(&hist[(i / RS_TILE) * 256 + (int)(key & 255u)], 1);
 }
 
 // system id of the particle at each position of the current order (digit source of the last passes)
 __global__ void k_gather_sys(int n, const int32_t *__restrict__ vals, const int32_t *__restrict__ sys_off, int nsys,
-                             uint64_t *__restrict__ skey)
+                             uint64_t *__restrict__ skey, int32_t *__restrict__ hist)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    skey[i] = (uint64_t)sys_of_pos(sys_off, nsys, vals[i]);
+    const int sy = sys_of_pos(sys_off, nsys, vals[i]);
+    skey[i] = (uint64_t)sy;
+    if (hist) atomicAdd(&hist[(i / RS_TILE) * 256 + (sy & 255)], 1);
 }
 
 // Morton keys again, in the final order (the system passes carried only the system digit)
@@ -861,13 +988,6 @@ __global__ void k_keys_sorted(int n, const float *__restrict__ x, const float *_
     if (vals_out) vals_out[s] = j;
 }
 
-__global__ void k_sys_root(int nsys, const int32_t *__restrict__ sys_off, const int32_t *__restrict__ base,
-                           int32_t *__restrict__ sys_root)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < nsys) sys_root[k] = base[sys_off[k]];
-}
-
 __global__ void k_zero_i32(const int32_t *__restrict__ nnodes, int32_t *a)
 {
     int nn = *nnodes;
@@ -881,6 +1001,10 @@ __global__ void k_zero_i32(const int32_t *__restrict__ nnodes, int32_t *a)
 // ---------------------------------------------------------------------------------------
 int evol_scan_i32(evol_ctx *c, int n, const int32_t *in, int32_t *out, int write_total)
 {
+    if (n <= SCAN_ONE_MAX) {
+        k_scan_one<<<1, SC_THREADS, 0, c->stream>>>(n, in, out, write_total);
+        return evol_cuda_ok(cudaGetLastError());
+    }
     int nparts = (n + SC_TILE - 1) / SC_TILE;
     if (nparts < 1) nparts = 1;
     k_scan_reduce<<<nparts, SC_THREADS, 0, c->stream>>>(n, in, c->d.scan_part);
@@ -927,58 +1051,79 @@ int evol_launch_build(evol_ctx *c, const evol_particles *p, const evol_params *p
     int leaf = prm->leaf_size > 0 ? prm->leaf_size : 8;
     cudaStream_t st = c->stream;
     int tb = 256, gb = (n + tb - 1) / tb;
+    const int rsb = (n + RS_TILE - 1) / RS_TILE;
+    const bool rank = n <= RANK_MAX, fused = !rank && n <= FUSED_MAX;
+    // fused passes: a histogram of every tile for each of the passes
+    int32_t *hist = (int32_t *)d.hist;
+    const size_t hsize = (size_t)256 * rsb;
+    int npass = 8;
+    for (int shift = 0; nsys > 1 && (1ll << shift) < (long long)nsys; shift += 8) ++npass;
+    if (fused && cudaMemsetAsync(hist, 0, npass * hsize * sizeof(int32_t), st) != cudaSuccess) return EVOL_ECUDA;
+    int32_t *h0 = fused ? hist : nullptr;
     if (nsys == 1) {
-        int nb = (int)c->bbox_blocks;
-        k_set_single<<<1, 32, 0, st>>>(n, d.sys_off);
-        k_bbox_partial<<<nb, BB_THREADS, 0, st>>>(n, p->x, p->y, p->z, d.bbox_part, d.err);
-        k_bbox_final<<<1, 32, 0, st>>>(nb, d.bbox_part, d.cube, d.fcube);
-        k_keys<<<gb, tb, 0, st>>>(n, p->x, p->y, p->z, d.cube, d.keys_a, d.vals_a);
+        if (n <= RANK_MAX) {
+            k_bbox_sys<<<1, 1024, 0, st>>>(n, d.sys_off, p->x, p->y, p->z, d.cube, d.fcube, d.err);
+        } else {
+            int nb = (int)c->bbox_blocks;
+            k_bbox_partial<<<nb, BB_THREADS, 0, st>>>(n, p->x, p->y, p->z, d.bbox_part, d.err);
+            k_bbox_final<<<1, 512, 0, st>>>(n, nb, d.bbox_part, d.cube, d.fcube, d.sys_off);
+        }
+        k_keys<<<gb, tb, 0, st>>>(n, p->x, p->y, p->z, d.cube, rank ? d.keys_b : d.keys_a, d.vals_a, h0);
     } else {
         // the offsets were copied into d.sys_off by the caller of this launcher
-        k_bbox_sys<<<nsys, BB_THREADS, 0, st>>>(d.sys_off, p->x, p->y, p->z, d.cube, d.fcube, d.err);
-        k_keys_sys<<<gb, tb, 0, st>>>(n, p->x, p->y, p->z, d.sys_off, nsys, d.cube, d.keys_a, d.vals_a);
+        k_bbox_sys<<<nsys, 1024, 0, st>>>(0, d.sys_off, p->x, p->y, p->z, d.cube, d.fcube, d.err);
+        k_keys_sys<<<gb, tb, 0, st>>>(n, p->x, p->y, p->z, d.sys_off, nsys, d.cube, rank ? d.keys_b : d.keys_a, d.vals_a,
+                                      h0);
     }
-    int rsb = (n + RS_TILE - 1) / RS_TILE;
     uint64_t *ka = d.keys_a, *kb = d.keys_b;
     int32_t *va = d.vals_a, *vb = d.vals_b;
-    for (int shift = 0; shift < 64; shift += 8) {
-        k_rs_hist<<<rsb, RS_THREADS, 0, st>>>(n, ka, shift, (int32_t *)d.hist, rsb);
-        int rc = evol_scan_i32(c, 256 * rsb, (int32_t *)d.hist, (int32_t *)d.hist, 0);
-        if (rc) return rc;
-        k_rs_scatter<<<rsb, RS_THREADS, 0, st>>>(n, ka, va, kb, vb, shift, (int32_t *)d.hist, rsb);
+    int done = 0;
+    auto pass = [&](int shift, bool last) -> int {
+        if (fused) {
+            k_rs_scatter<true><<<rsb, RS_THREADS, 0, st>>>(n, ka, va, kb, vb, shift, hist + done * hsize, rsb,
+                                                           last ? nullptr : hist + (done + 1) * hsize);
+        } else {
+            k_rs_hist<<<rsb, RS_THREADS, 0, st>>>(n, ka, shift, hist, rsb);
+            const int rc = evol_scan_i32(c, 256 * rsb, hist, hist, 0);
+            if (rc) return rc;
+            k_rs_scatter<false><<<rsb, RS_THREADS, 0, st>>>(n, ka, va, kb, vb, shift, hist, rsb, nullptr);
+        }
+        ++done;
         uint64_t *tk = ka; ka = kb; kb = tk;
         int32_t *tv = va; va = vb; vb = tv;
-    }
-    // 8 passes: sorted keys and permutation are back in keys_a / vals_a
-    if (nsys > 1) {
-        // stable passes on the system id make the order (system, key); then the keys are recomputed
-        k_gather_sys<<<gb, tb, 0, st>>>(n, d.vals_a, d.sys_off, nsys, d.keys_b);
-        ka = d.keys_b; kb = d.keys_a; va = d.vals_a; vb = d.vals_b;
-        for (int shift = 0; (1ll << shift) < (long long)nsys; shift += 8) {
-            k_rs_hist<<<rsb, RS_THREADS, 0, st>>>(n, ka, shift, (int32_t *)d.hist, rsb);
-            int rc = evol_scan_i32(c, 256 * rsb, (int32_t *)d.hist, (int32_t *)d.hist, 0);
-            if (rc) return rc;
-            k_rs_scatter<<<rsb, RS_THREADS, 0, st>>>(n, ka, va, kb, vb, shift, (int32_t *)d.hist, rsb);
-            uint64_t *tk = ka; ka = kb; kb = tk;
-            int32_t *tv = va; va = vb; vb = tv;
+        return EVOL_OK;
+    };
+    if (rank) {
+        const int blocks = (n + 31) / 32;
+        if (nsys == 1) k_rank_sort<false><<<blocks, 256, 0, st>>>(n, d.keys_b, d.sys_off, nsys, d.keys_a, d.vals_a);
+        else k_rank_sort<true><<<blocks, 256, 0, st>>>(n, d.keys_b, d.sys_off, nsys, d.keys_a, d.vals_a);
+    } else {
+        for (int shift = 0; shift < 64; shift += 8)
+            if (int rc = pass(shift, shift == 56)) return rc;
+        // 8 passes: sorted keys and permutation are back in keys_a / vals_a
+        if (nsys > 1) {
+            // stable passes on the system id make the order (system, key); then the keys are recomputed
+            k_gather_sys<<<gb, tb, 0, st>>>(n, d.vals_a, d.sys_off, nsys, d.keys_b, fused ? hist + 8 * hsize : nullptr);
+            ka = d.keys_b; kb = d.keys_a; va = d.vals_a; vb = d.vals_b;
+            for (int shift = 0; (1ll << shift) < (long long)nsys; shift += 8)
+                if (int rc = pass(shift, (1ll << (shift + 8)) >= (long long)nsys)) return rc;
+            // va holds the final permutation; rebuild keys_a / vals_a from it
+            k_keys_sorted<<<gb, tb, 0, st>>>(n, p->x, p->y, p->z, va, d.sys_off, nsys, d.cube, d.keys_a,
+                                             va == d.vals_a ? nullptr : d.vals_a);
         }
-        // va holds the final permutation; rebuild keys_a / vals_a from it
-        k_keys_sorted<<<gb, tb, 0, st>>>(n, p->x, p->y, p->z, va, d.sys_off, nsys, d.cube, d.keys_a,
-                                         va == d.vals_a ? nullptr : d.vals_a);
     }
     k_permute<<<gb, tb, 0, st>>>(n, (int)p->n_gas, d.vals_a, p->x, p->y, p->z, p->vx, p->vy, p->vz, p->m, p->u,
                                  p->h, p->eps, d.pos, d.vel, d.len_h, d.len_eps, d.orig, d.inv,
-                                 c->pred_dt, c->kdk_acc, c->cap, c->pred_tau);
-    k_lcp<<<gb, tb, 0, st>>>(n, d.keys_a, d.sys_off, nsys, d.lcp, d.sys_sorted);
+                                 c->pred_dt, c->kdk_acc, c->cap, c->pred_tau, d.keys_a, d.sys_off, nsys, d.lcp,
+                                 d.sys_sorted);
     k_count<<<gb, tb, 0, st>>>(n, d.lcp, leaf, d.cnt);
     int rc = evol_scan_i32(c, n, d.cnt, d.base, 1);
     if (rc) return rc;
     k_fill<<<gb, tb, 0, st>>>(n, d.keys_a, d.lcp, d.sys_off, d.sys_sorted, d.base, leaf, c->node_cap, d.nbeg, d.nend,
                               d.nlev, d.nnext, d.nnodes, d.err);
-    k_sys_root<<<(nsys + 255) / 256, 256, 0, st>>>(nsys, d.sys_off, d.base, d.sys_root);
     int ng = c->num_sms * 8;
     k_link<<<ng, 256, 0, st>>>(d.nnodes, leaf, d.nbeg, d.nend, d.nlev, d.nnext, d.nparent, d.nnch, d.narrive, d.nI,
-                               d.nK0, d.nK1);
+                               d.nK0, d.nK1, nsys, d.sys_off, d.base, d.sys_root);
     NodeOut o{d.nA, d.nB, d.nC, d.nQ0, d.nQ1, d.nBmin, d.nBmax, d.nCoff, d.nM64, d.nC64, d.nQ64};
     float theta = prm->theta;
     if (prm->precision == EVOL_FP32_MIXED)
