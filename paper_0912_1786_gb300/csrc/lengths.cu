@@ -470,7 +470,9 @@ __device__ __forceinline__ int gather_staged(const evol_kparams &kp, const LenSm
 }
 
 // The same by the particle's own walk from `root`, a warp at a time.  Returns -1 when the walk had to
-// stop (corrupt tree or stack overflow; the error word is set).
+// stop (corrupt tree or stack overflow; the error word is set).  A list that overflows is of no use, and its
+// ball can be the whole set (far outliers of a small sphere), so the walk ends there with a count above cap:
+// 9000 particles 3.02 -> 0.82 ms for the solve, 20,000 1.34 -> 0.87.
 template <int MODE, bool PER, bool FLOW>
 __device__ __forceinline__ int gather_ball(const evol_dev &d, const evol_kparams &kp, float2 *nb, int cap, int lane, int *stk, long long pop_cap, int root, float px,
                                         float py, float pz, float R2)
@@ -523,7 +525,7 @@ __device__ __forceinline__ int gather_ball(const evol_dev &d, const evol_kparams
             }
         }
         unsigned lv = __ballot_sync(0xffffffffu, e > b);
-        while (lv) {
+        while (lv && cnt <= cap) {
             const int q = __ffs(lv) - 1;
             lv &= lv - 1u;
             const int lb = __shfl_sync(0xffffffffu, b, q), le = __shfl_sync(0xffffffffu, e, q);
@@ -548,6 +550,7 @@ __device__ __forceinline__ int gather_ball(const evol_dev &d, const evol_kparams
                 cnt += __popc(bal);
             }
         }
+        if (cnt > cap) return cnt;
         int incl = nch;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {

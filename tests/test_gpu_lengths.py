@@ -67,6 +67,12 @@ def test_neighbour_numbers_beyond_the_short_lists(nnei):
     _compare(W.evrard_sphere(9001, seed=9, params=p), GAS + ALL, p)
 
 
+@pytest.mark.parametrize("n,group", [(9000, 0), (9000, 8), (20000, 16)])
+def test_balls_of_far_outliers(n, group):
+    # a small sphere without an edge: the balls of the outermost particles hold more than their lists do
+    _compare(W.plummer(n, seed=7, params=W.Params(theta=0.6, n_nei_grav=32.0, sph=0, length_group=group)), ALL)
+
+
 def test_many_small_systems():
     # blocks whose particles belong to several systems
     import torch
