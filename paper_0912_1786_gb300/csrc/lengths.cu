@@ -472,7 +472,7 @@ __device__ __forceinline__ int gather_staged(const evol_kparams &kp, const LenSm
 // The same by the particle's own walk from `root`, a warp at a time.  Returns -1 when the walk had to
 // stop (corrupt tree or stack overflow; the error word is set).  A list that overflows is of no use, and its
 // ball can be the whole set (far outliers of a small sphere), so the walk ends there with a count above cap:
-// 9000 particles 3.02 -> 0.82 ms for the solve, 20,000 1.34 -> 0.87.
+// 9000 particles 3.02 -> 0.82 ms for the solve, 20,000 1.34 -> 0.87 (0.47 and 0.69 with the turns below).
 template <int MODE, bool PER, bool FLOW>
 __device__ __forceinline__ int gather_ball(const evol_dev &d, const evol_kparams &kp, float2 *nb, int cap, int lane, int *stk, long long pop_cap, int root, float px,
                                         float py, float pz, float R2)
@@ -524,31 +524,39 @@ __device__ __forceinline__ int gather_ball(const evol_dev &d, const evol_kparams
                 }
             }
         }
-        unsigned lv = __ballot_sync(0xffffffffu, e > b);
-        while (lv && cnt <= cap) {
-            const int q = __ffs(lv) - 1;
-            lv &= lv - 1u;
-            const int lb = __shfl_sync(0xffffffffu, b, q), le = __shfl_sync(0xffffffffu, e, q);
-            for (int c0 = lb; c0 < le; c0 += 32) {
-                const int j = c0 + lane;
-                bool in = false;
-                float r2 = 0.f, m = 0.f;
-                if (j < le) {
-                    const float4 p = gas_lists<MODE>(kp) ? d.gpos[j] : d.pos[j];
-                    const float dx = image<PER>(px - p.x, kp, 0), dy = image<PER>(py - p.y, kp, 1),
-                                dz = image<PER>(pz - p.z, kp, 2);
-                    r2 = dx * dx + dy * dy + dz * dz;
-                    in = r2 < R2;
-                    m = p.w;
-                }
-                const unsigned bal = __ballot_sync(0xffffffffu, in);
-                if (in) {
-                    const int o = cnt + __popc(bal & ltmask);
-                    if (o < cap)
-                        nb[o] = make_float2(sqrtf(r2), FLOW ? __int_as_float(gas_lists<MODE>(kp) ? d.glist[j] : j) : m);
-                }
-                cnt += __popc(bal);
+        // the leaves' particles one after the other, 32 a turn (a leaf a turn took four times as many turns,
+        // each a round trip to L2, with leaves of eight)
+        int li = e - b;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, li, o);
+            if (lane >= o) li += t;
+        }
+        const int lt = __shfl_sync(0xffffffffu, li, 31), l0 = e - li;      // position of entry t: l0 + t
+        for (int t0 = 0; t0 < lt && cnt <= cap; t0 += 32) {
+            const int t = t0 + lane;
+            int q = 0;                          // the leaf of entry t: the first with more entries up to its end
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, li, q + o - 1) <= t) q += o;
+            const int j = __shfl_sync(0xffffffffu, l0, q & 31) + t;
+            bool in = false;
+            float r2 = 0.f, m = 0.f;
+            if (t < lt) {
+                const float4 p = gas_lists<MODE>(kp) ? d.gpos[j] : d.pos[j];
+                const float dx = image<PER>(px - p.x, kp, 0), dy = image<PER>(py - p.y, kp, 1),
+                            dz = image<PER>(pz - p.z, kp, 2);
+                r2 = dx * dx + dy * dy + dz * dz;
+                in = r2 < R2;
+                m = p.w;
             }
+            const unsigned bal = __ballot_sync(0xffffffffu, in);
+            if (in) {
+                const int o = cnt + __popc(bal & ltmask);
+                if (o < cap)
+                    nb[o] = make_float2(sqrtf(r2), FLOW ? __int_as_float(gas_lists<MODE>(kp) ? d.glist[j] : j) : m);
+            }
+            cnt += __popc(bal);
         }
         if (cnt > cap) return cnt;
         int incl = nch;
