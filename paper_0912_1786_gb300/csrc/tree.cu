@@ -627,280 +627,387 @@ __global__ void k_link(const int32_t *__restrict__ nnodes, int leaf, const int32
 // Moments, leaf-up.  A leaf sums its particles; the last child to finish a parent (atomic
 // arrival count) combines the children with the parallel-axis shift of the quadrupole.
 //
-// FP32 (plain) moments take every position relative to the node's geometric centre (exact in
-// double: a dyadic point of the root cube), so the centre of mass and the quadrupole carry
-// rounding on the scale of the node, not of the coordinates; a parent combines its children's
-// centre-of-mass offsets shifted by the (power-of-two) difference of the two centres, which is
-// exact in float.  The absolute centre of mass is formed once, in double, when the node is
-// written.  FP64 (mixed) moments use absolute coordinates.
+// FP32 (plain) moments take every position relative to the node's geometric centre (a dyadic point of the
+// root cube, see Centre), so the centre of mass and the quadrupole carry rounding on the scale of the
+// node, not of the coordinates; a parent combines its children's centre-of-mass offsets shifted by the
+// (power-of-two) difference of the two centres, which is exact in float.  The absolute centre of mass
+// is formed once, by k_node_geometry.  FP64 (mixed) moments use absolute coordinates.
 // ---------------------------------------------------------------------------------------
-template <typename T>
-struct Mom {
-    T M, c[3], q[6];       // mass, centre of mass (FP32: offset from the node centre), traceless
-                           // quadrupole about it (xx yy zz xy xz yz)
-};
-
 struct NodeOut {
     float4 *nA, *nB, *nC, *nQ0, *nQ1, *bmin, *bmax, *coff;
     double *M64, *C64, *Q64;
 };
 
-// geometric centre of the node whose first key is key0 at level lev (exact in double)
-__device__ __forceinline__ void node_centre(const double *__restrict__ cube, uint64_t key0, int lev, double cg[3])
+// bits 0, 3, 6, ... of v, packed (the inverse of spread3)
+__device__ __forceinline__ unsigned compact3(uint64_t v)
 {
-    double side = ldexp(cube[3], -lev);
-    uint64_t qa[3] = {0, 0, 0};
-    for (int l = 1; l <= lev; ++l) {
-        unsigned dg = (unsigned)(key0 >> (3 * (EVOL_MAXLEVEL - l))) & 7u;
-        qa[0] = (qa[0] << 1) | ((dg >> 2) & 1u);
-        qa[1] = (qa[1] << 1) | ((dg >> 1) & 1u);
-        qa[2] = (qa[2] << 1) | (dg & 1u);
-    }
-    for (int a = 0; a < 3; ++a) cg[a] = cube[a] + ((double)qa[a] + 0.5) * side;
+    v &= 0x1249249249249249ull;
+    v = (v | (v >> 2)) & 0x10c30c30c30c30c3ull;
+    v = (v | (v >> 4)) & 0x100f00f00f00f00full;
+    v = (v | (v >> 8)) & 0x1f0000ff0000ffull;
+    v = (v | (v >> 16)) & 0x1f00000000ffffull;
+    return (unsigned)(v | (v >> 32)) & 0x1fffffu;
 }
 
-template <typename T>
-__device__ void write_node(const NodeOut &o, int id, const Mom<T> &mm, float3 lo, float3 hi, int hasgas, int lev,
-                           const double cg[3], double side, float theta, bool mixed)
+// cell index along axis a (0: x) of the node whose first key is key0 at level lev
+__device__ __forceinline__ unsigned cell_index(uint64_t key0, int lev, int a)
 {
-    constexpr bool rel = sizeof(T) == sizeof(float);
-    double com[3], dd = 0.0;
-    for (int a = 0; a < 3; ++a) {
-        const double off = rel ? (double)mm.c[a] : (double)mm.c[a] - cg[a];
-        com[a] = rel ? cg[a] + off : (double)mm.c[a];
-        dd += off * off;
-    }
-    float delta = (float)sqrt(dd);
-    float l = (float)side;
-    float ropen = theta > 0.f ? l / theta + delta : INFINITY;
-    o.nA[id] = make_float4((float)com[0], (float)com[1], (float)com[2], ropen * ropen);
-    float4 bb = make_float4(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z), hasgas ? 0.f : -1.f);
-    o.nB[id] = bb;
-    o.nC[id] = make_float4(0.5f * (hi.x - lo.x), 0.5f * (hi.y - lo.y), 0.5f * (hi.z - lo.z), 0.f);
-    o.nQ0[id] = make_float4((float)mm.q[0], (float)mm.q[1], (float)mm.q[2], (float)mm.M);
-    o.nQ1[id] = make_float4((float)mm.q[3], (float)mm.q[4], (float)mm.q[5], delta);
-    o.bmin[id] = make_float4(lo.x, lo.y, lo.z, (float)hasgas);
-    o.bmax[id] = make_float4(hi.x, hi.y, hi.z, 0.f);
-    if (rel) o.coff[id] = make_float4((float)mm.c[0], (float)mm.c[1], (float)mm.c[2], (float)mm.M);
-    if (mixed) {
-        o.M64[id] = (double)mm.M;
-        for (int a = 0; a < 3; ++a) o.C64[3 * id + a] = (double)mm.c[a];
-        for (int a = 0; a < 6; ++a) o.Q64[6 * id + a] = (double)mm.q[a];
-    }
+    return compact3(key0 >> (3 * (EVOL_MAXLEVEL - lev)) >> (2 - a));
 }
 
-template <typename T>
-__device__ void leaf_moments(int b, int e, int n_gas, const float4 *__restrict__ pos, const int32_t *__restrict__ orig,
-                             const double cg[3], Mom<T> &mm, float3 &lo, float3 &hi, int &hasgas)
+// A node's geometric centre along one axis, as the sum of two floats.  The cube's corner is a float, and the
+// centre's offset from it an odd number of 22 bits times a power of two, so the sum of the two in hi + lo is
+// exact, and a float minus the centre is right to the rounding of the result, without double arithmetic.
+struct Centre {
+    float hi, lo;
+};
+
+__device__ __forceinline__ Centre two_sum(float a, float b)
 {
-    constexpr bool rel = sizeof(T) == sizeof(float);
-    T M = 0, s0 = 0, s1 = 0, s2 = 0;
-    lo = make_float3(INFINITY, INFINITY, INFINITY);
-    hi = make_float3(-INFINITY, -INFINITY, -INFINITY);
-    hasgas = 0;
-    auto coord = [&](float x, int a) -> T { return rel ? (T)((double)x - cg[a]) : (T)x; };
-    for (int s = b; s < e; ++s) {
-        float4 p = pos[s];
-        M += (T)p.w;
-        s0 += (T)p.w * coord(p.x, 0);
-        s1 += (T)p.w * coord(p.y, 1);
-        s2 += (T)p.w * coord(p.z, 2);
-        lo.x = fminf(lo.x, p.x); lo.y = fminf(lo.y, p.y); lo.z = fminf(lo.z, p.z);
-        hi.x = fmaxf(hi.x, p.x); hi.y = fmaxf(hi.y, p.y); hi.z = fmaxf(hi.z, p.z);
-        if (orig[s] < n_gas) hasgas = 1;
-    }
-    mm.M = M;
-    if (M > 0) {
-        mm.c[0] = s0 / M; mm.c[1] = s1 / M; mm.c[2] = s2 / M;
-    } else {
-        mm.c[0] = coord(0.5f * (lo.x + hi.x), 0);
-        mm.c[1] = coord(0.5f * (lo.y + hi.y), 1);
-        mm.c[2] = coord(0.5f * (lo.z + hi.z), 2);
-    }
-    for (int a = 0; a < 6; ++a) mm.q[a] = 0;
-    for (int s = b; s < e; ++s) {
-        float4 p = pos[s];
-        T d0 = coord(p.x, 0) - mm.c[0], d1 = coord(p.y, 1) - mm.c[1], d2 = coord(p.z, 2) - mm.c[2];
-        T r2 = d0 * d0 + d1 * d1 + d2 * d2, w = (T)p.w;
-        mm.q[0] += w * (3 * d0 * d0 - r2);
-        mm.q[1] += w * (3 * d1 * d1 - r2);
-        mm.q[2] += w * (3 * d2 * d2 - r2);
-        mm.q[3] += w * 3 * d0 * d1;
-        mm.q[4] += w * 3 * d0 * d2;
-        mm.q[5] += w * 3 * d1 * d2;
-    }
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
 }
 
-// child c's moments; FP32: its centre-of-mass offset re-expressed about the parent's centre.  A
-// child cell is one level below its parent (a cell with one non-empty octant still has that octant
-// as its child), so its centre is the parent's centre moved by a quarter of the parent's side
-// along each axis, in the direction the child's octal digit gives: a power of two, exact in float.
-template <typename T>
-__device__ void load_child(const NodeOut &o, int c, float side_p, const uint64_t *__restrict__ keys,
-                           const int32_t *__restrict__ nbeg, const int32_t *__restrict__ nlev, Mom<T> &mm,
-                           float3 &lo, float3 &hi, int &hasgas, bool mixed)
+__device__ __forceinline__ Centre node_centre(float corner, float side, unsigned cell, int lev)
 {
-    constexpr bool rel = sizeof(T) == sizeof(float);
-    float4 bl = __ldcg(&o.bmin[c]), bh = __ldcg(&o.bmax[c]);
-    lo = make_float3(bl.x, bl.y, bl.z);
-    hi = make_float3(bh.x, bh.y, bh.z);
-    hasgas = bl.w != 0.f;
-    float4 Q0, Q1;
-    if (mixed) {
-        mm.M = (T)__ldcg(&o.M64[c]);
-        for (int a = 0; a < 3; ++a) mm.c[a] = (T)__ldcg(&o.C64[3 * c + a]);
-        for (int a = 0; a < 6; ++a) mm.q[a] = (T)__ldcg(&o.Q64[6 * c + a]);
-        return;
-    }
-    Q0 = __ldcg(&o.nQ0[c]);
-    Q1 = __ldcg(&o.nQ1[c]);
-    mm.q[0] = (T)Q0.x; mm.q[1] = (T)Q0.y; mm.q[2] = (T)Q0.z;
-    mm.q[3] = (T)Q1.x; mm.q[4] = (T)Q1.y; mm.q[5] = (T)Q1.z;
-    if (rel) {
-        const float4 co = __ldcg(&o.coff[c]);
-        const int lc = __ldcg(&nlev[c]);
-        const unsigned dg = (unsigned)(__ldcg(&keys[__ldcg(&nbeg[c])]) >> (3 * (EVOL_MAXLEVEL - lc))) & 7u;
-        const float q = 0.25f * side_p;
-        mm.M = (T)co.w;
-        mm.c[0] = (T)co.x + (T)((dg & 4u) ? q : -q);
-        mm.c[1] = (T)co.y + (T)((dg & 2u) ? q : -q);
-        mm.c[2] = (T)co.z + (T)((dg & 1u) ? q : -q);
-    } else {
-        const float4 A = __ldcg(&o.nA[c]);
-        mm.M = (T)Q0.w;
-        mm.c[0] = (T)A.x; mm.c[1] = (T)A.y; mm.c[2] = (T)A.z;
-    }
+    return two_sum(corner, (float)(2u * cell + 1u) * ldexpf(side, -lev - 1));
 }
 
-template <typename T>
-__device__ void combine(const NodeOut &o, int id, int nch, const int32_t *__restrict__ nnext, const double cgp[3],
-                        float side_p, const uint64_t *__restrict__ keys, const int32_t *__restrict__ nbeg,
-                        const int32_t *__restrict__ nlev, Mom<T> &mm, float3 &lo, float3 &hi, int &hasgas, bool mixed)
+// x minus the centre
+__device__ __forceinline__ float from_centre(float x, const Centre &c)
 {
-    constexpr bool rel = sizeof(T) == sizeof(float);
-    Mom<T> ch[8];
-    lo = make_float3(INFINITY, INFINITY, INFINITY);
-    hi = make_float3(-INFINITY, -INFINITY, -INFINITY);
-    hasgas = 0;
-    T M = 0, s[3] = {0, 0, 0};
-    int c = id + 1;
-    for (int k = 0; k < nch; ++k) {
-        float3 cl, chh;
-        int cg;
-        load_child(o, c, side_p, keys, nbeg, nlev, ch[k], cl, chh, cg, mixed);
-        lo.x = fminf(lo.x, cl.x); lo.y = fminf(lo.y, cl.y); lo.z = fminf(lo.z, cl.z);
-        hi.x = fmaxf(hi.x, chh.x); hi.y = fmaxf(hi.y, chh.y); hi.z = fmaxf(hi.z, chh.z);
-        hasgas |= cg;
-        M += ch[k].M;
-        for (int a = 0; a < 3; ++a) s[a] += ch[k].M * ch[k].c[a];
-        c = nnext[c];
-    }
-    mm.M = M;
-    float cen[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
-    for (int a = 0; a < 3; ++a) mm.c[a] = M > 0 ? s[a] / M : (rel ? (T)((double)cen[a] - cgp[a]) : (T)cen[a]);
-    for (int a = 0; a < 6; ++a) mm.q[a] = 0;
-    for (int j = 0; j < nch; ++j) {
-        T d0 = ch[j].c[0] - mm.c[0], d1 = ch[j].c[1] - mm.c[1], d2 = ch[j].c[2] - mm.c[2];
-        T r2 = d0 * d0 + d1 * d1 + d2 * d2, w = ch[j].M;
-        mm.q[0] += ch[j].q[0] + w * (3 * d0 * d0 - r2);
-        mm.q[1] += ch[j].q[1] + w * (3 * d1 * d1 - r2);
-        mm.q[2] += ch[j].q[2] + w * (3 * d2 * d2 - r2);
-        mm.q[3] += ch[j].q[3] + w * 3 * d0 * d1;
-        mm.q[4] += ch[j].q[4] + w * 3 * d0 * d2;
-        mm.q[5] += ch[j].q[5] + w * 3 * d1 * d2;
-    }
+    const Centre d = two_sum(x, -c.hi);
+    return __fadd_rn(d.hi, __fsub_rn(d.lo, c.lo));
 }
 
-template <typename T>
-__global__ void k_moments(const int32_t *__restrict__ nnodes, int n_gas, const int32_t *__restrict__ nbeg,
-                          const int32_t *__restrict__ nend, const int32_t *__restrict__ nlev,
-                          const int32_t *__restrict__ nnext, const int32_t *__restrict__ nparent,
-                          const int32_t *__restrict__ nnch, int32_t *__restrict__ narrive,
-                          const float4 *__restrict__ pos, const int32_t *__restrict__ orig,
-                          const uint64_t *__restrict__ keys, const double *__restrict__ cube,
-                          const int32_t *__restrict__ sys_sorted, float theta, NodeOut o, int mixed, int *err)
+// The totals over an octet's eight lanes of eight values each: lane k gets value k's (seven exchanges instead
+// of 24).
+template <typename T, typename Op>
+__device__ __forceinline__ T octet_reduce(T (&v)[8], int sub, Op op)
 {
-    int nn = *nnodes;
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nn; id += gridDim.x * blockDim.x) {
-        if (nnch[id] != 0) continue;
-        Mom<T> mm;
-        float3 lo, hi;
-        int hg;
-        const double *cb = cube + 4 * sys_sorted[nbeg[id]];
-        double cg[3];
-        node_centre(cb, keys[nbeg[id]], nlev[id], cg);
-        leaf_moments<T>(nbeg[id], nend[id], n_gas, pos, orig, cg, mm, lo, hi, hg);
-        write_node<T>(o, id, mm, lo, hi, hg, nlev[id], cg, ldexp(cb[3], -nlev[id]), theta, mixed != 0);
-        __threadfence();
-        int p = nparent[id];
-        for (int climb = 0; p >= 0 && p < nn; ++climb) {
-            if (climb > EVOL_MAXLEVEL + 1) {     // deeper than the tree can be: corrupt parents
-                evol_flag(err, EVOL_ETIMEOUT);
-                break;
-            }
-            int old = atomicAdd(&narrive[p], 1);
-            if (old != nnch[p] - 1) break;
-            __threadfence();
-            const double *cbp = cube + 4 * sys_sorted[nbeg[p]];
-            double cgp[3];
-            node_centre(cbp, keys[nbeg[p]], nlev[p], cgp);
-            combine<T>(o, p, nnch[p], nnext, cgp, (float)ldexp(cbp[3], -nlev[p]), keys, nbeg, nlev, mm, lo, hi, hg,
-                       mixed != 0);
-            write_node<T>(o, p, mm, lo, hi, hg, nlev[p], cgp, ldexp(cbp[3], -nlev[p]), theta, mixed != 0);
-            __threadfence();
-            p = nparent[p];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        const bool up = sub & o;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const T give = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
+            v[k] = op(keep, __shfl_xor_sync(0xffffffffu, give, o));
         }
+    }
+    return v[0];
+}
+
+// The same of four values: lanes k and k + 4 get value k's.
+template <typename T>
+__device__ __forceinline__ T octet_sum4(T (&v)[4], int sub)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], 4);
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) {
+        const bool up = sub & o;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const T give = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    return v[0];
+}
+
+struct Links {
+    const int32_t *nnodes, *nparent, *nnch;
+    const int4 *nI, *nK0, *nK1;
+    int32_t *narrive;
+    int *err;
+};
+
+// Leaf-up pass over the tree: eight lanes to a node, in a leaf a lane to a particle, above a lane to a child.
+// The octet that completes a parent goes on with it, the others end; a warp starts on the leaves among
+// its next nodes, four at a time.  leaf(id, I) and node(id, I, child, pre) form and store a node's values
+// (id < 0: nothing to do; all 32 lanes call them); pre(child, level) is read ahead of the parent's
+// completion, as are all its links: what remains of a level is the chain store, fence, count, load of the
+// children's values.  The counts are left at zero for the next pass.
+template <typename Leaf, typename Pre, typename Node>
+__device__ __forceinline__ void leaf_up(const Links &L, Leaf leaf, Pre pre, Node node)
+{
+    const int nn = *L.nnodes, lane = threadIdx.x & 31, sub = lane & 7;
+    const int warps = gridDim.x * (blockDim.x >> 5), wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    // nodes a turn: 32, fewer where that leaves warps without any
+    const int per = min(32, (nn / warps + 4) & ~3);
+    for (int base = wid * per; base < nn; base += warps * per) {
+        unsigned todo = __ballot_sync(0xffffffffu, lane < per && base + lane < nn && L.nnch[base + lane] == 0);
+        while (todo) {
+            int id = -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if ((lane >> 3) == q && todo) id = base + __ffs(todo) - 1;
+                todo &= todo - 1u;
+            }
+            leaf(id, id >= 0 ? L.nI[id] : make_int4(0, 0, 0, 0));
+            for (int climb = 0;; ++climb) {
+                if (climb > EVOL_MAXLEVEL + 1) {     // deeper than the tree can be: corrupt parents
+                    if (lane == 0) evol_flag(L.err, EVOL_ETIMEOUT);
+                    break;
+                }
+                int p = id >= 0 ? L.nparent[id] : -1;
+                if (p >= nn) p = -1;
+                int4 I = make_int4(0, 0, 0, 0);
+                int nch = 0, c = -1;
+                if (p >= 0) {
+                    I = L.nI[p];
+                    nch = L.nnch[p];
+                    c = reinterpret_cast<const int *>(sub < 4 ? L.nK0 : L.nK1)[4 * (size_t)p + (sub & 3)];
+                }
+                const auto ahead = pre(c, (I.x & 0xff) + 1);
+                __threadfence();
+                __syncwarp();
+                int old = -1;
+                if (p >= 0 && sub == 0) old = atomicAdd(&L.narrive[p], 1);
+                old = __shfl_sync(0xffffffffu, old, lane & 24);
+                const bool last = p >= 0 && old == nch - 1;
+                if (last && sub == 0) L.narrive[p] = 0;
+                if (!__any_sync(0xffffffffu, last)) break;
+                __threadfence();
+                __syncwarp();
+                id = last ? p : -1;
+                node(id, I, last ? c : -1, ahead);
+            }
+        }
+    }
+}
+
+// Moments of every node: mass, centre of mass (FP32: its offset from the node's centre), quadrupole about it, and
+// the particles' box.  Bound by the chain of dependent steps from the leaves to the root, not by its reads.
+// A thread per node, its children one after the other and each in dependent loads, took 54 us with 1000
+// particles, 141 with 49 k and 962 with 3.1 M; this and k_node_geometry take 26, 58 and 274 (FP64 of 393 k:
+// 389 -> 184), k_node_lengths 13, 32 and 154 (26, 77 and 197).
+template <typename T>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 5)
+    k_moments(Links L, int n_gas, const float4 *__restrict__ pos, const int32_t *__restrict__ orig,
+              const uint64_t *__restrict__ keys, const float *__restrict__ fcube,
+              const int32_t *__restrict__ sys_sorted, NodeOut o)
+{
+    constexpr bool rel = sizeof(T) == sizeof(float);
+    const int lane = threadIdx.x & 31, sub = lane & 7, oct = lane & 24;
+    // an octet's node from its lanes' shares: mass and mass times position, box (lo, -hi, -gas), then the
+    // quadrupole shares that add_q makes about the centre of mass
+    auto finish = [&](int id, int lev, int beg, T (&ms)[4], float (&bx)[8], auto add_q) {
+        const T sum = octet_sum4(ms, sub);
+        const float bound = octet_reduce(bx, sub, [](float a, float b) { return fminf(a, b); });
+        const T M = __shfl_sync(0xffffffffu, sum, oct);
+        T c[3];
+        const T cv = sum / M;                      // lanes 1 .. 3
+#pragma unroll
+        for (int a = 0; a < 3; ++a) c[a] = __shfl_sync(0xffffffffu, cv, oct + 1 + a);
+        if (__any_sync(0xffffffffu, id >= 0 && !(M > 0))) {
+            // no mass: the middle of the box
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float lo = __shfl_sync(0xffffffffu, bound, oct + a), hi = -__shfl_sync(0xffffffffu, bound, oct + 3 + a);
+                if (id >= 0 && !(M > 0)) {
+                    if (rel) {
+                        const float *cb = fcube + 4 * sys_sorted[beg];
+                        const Centre cg = node_centre(cb[a], cb[3], cell_index(keys[beg], lev, a), lev);
+                        c[a] = (T)(0.5f * (from_centre(lo, cg) + from_centre(hi, cg)));
+                    } else {
+                        c[a] = (T)0.5 * ((T)lo + (T)hi);
+                    }
+                }
+            }
+        }
+        T q[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        add_q(c, q);
+        const T qv = octet_reduce(q, sub, [](T a, T b) { return a + b; });
+        if (id < 0) return;
+        float *qf = (float *)(sub >= 3 && sub < 6 ? o.nQ1 : o.nQ0) + 4 * (size_t)id;
+        if (sub < 7) qf[sub == 6 ? 3 : sub < 3 ? sub : sub - 3] = sub == 6 ? (float)M : (float)qv;
+        float *bf = (float *)(sub == 7 || (sub >= 3 && sub < 6) ? o.bmax : o.bmin) + 4 * (size_t)id;
+        bf[sub >= 6 ? 3 : sub < 3 ? sub : sub - 3] = sub == 7 ? 0.f : sub < 3 ? bound : 0.f - bound;
+        const T cs = sub == 0 ? c[0] : sub == 1 ? c[1] : sub == 2 ? c[2] : M;
+        if (rel) {
+            if (sub < 4) reinterpret_cast<float *>(o.coff)[4 * (size_t)id + sub] = (float)cs;
+        } else {
+            if (sub < 3) o.C64[3 * (size_t)id + sub] = (double)cs;
+            if (sub == 3) o.M64[id] = (double)cs;
+            if (sub < 6) o.Q64[6 * (size_t)id + sub] = (double)qv;
+        }
+    };
+    auto quad = [](T (&q)[8], T w, T d0, T d1, T d2) {
+        const T r2 = d0 * d0 + d1 * d1 + d2 * d2;
+        q[0] += w * (3 * d0 * d0 - r2);
+        q[1] += w * (3 * d1 * d1 - r2);
+        q[2] += w * (3 * d2 * d2 - r2);
+        q[3] += w * 3 * d0 * d1;
+        q[4] += w * 3 * d0 * d2;
+        q[5] += w * 3 * d1 * d2;
+    };
+    auto box = [](float (&bx)[8]) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) bx[k] = INFINITY;
+        bx[6] = bx[7] = 0.f;
+    };
+    leaf_up(
+        L,
+        [&](int id, const int4 &I) {
+            const int lev = I.x & 0xff, b = I.z, e = id >= 0 ? I.w : I.z;
+            Centre cg[3] = {};
+            if (rel) {
+                // axis a's on lane a, then to all
+                Centre m = {0.f, 0.f};
+                if (id >= 0 && sub < 3) {
+                    const float *cb = fcube + 4 * sys_sorted[b];
+                    m = node_centre(cb[sub], cb[3], cell_index(keys[b], lev, sub), lev);
+                }
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    cg[a] = {__shfl_sync(0xffffffffu, m.hi, oct + a), __shfl_sync(0xffffffffu, m.lo, oct + a)};
+            }
+            auto coord = [&](float x, int a) -> T { return rel ? (T)from_centre(x, cg[a]) : (T)x; };
+            T ms[4] = {0, 0, 0, 0};
+            float bx[8];
+            box(bx);
+            for (int s = b + sub; s < e; s += 8) {
+                const float4 p = pos[s];
+                if (orig[s] < n_gas) bx[6] = -1.f;
+                const T w = (T)p.w;
+                ms[0] += w;
+                ms[1] += w * coord(p.x, 0);
+                ms[2] += w * coord(p.y, 1);
+                ms[3] += w * coord(p.z, 2);
+                bx[0] = fminf(bx[0], p.x); bx[1] = fminf(bx[1], p.y); bx[2] = fminf(bx[2], p.z);
+                bx[3] = fminf(bx[3], -p.x); bx[4] = fminf(bx[4], -p.y); bx[5] = fminf(bx[5], -p.z);
+            }
+            finish(id, lev, b, ms, bx, [&](const T (&c)[3], T (&q)[8]) {
+                for (int s = b + sub; s < e; s += 8) {
+                    const float4 p = pos[s];
+                    quad(q, (T)p.w, coord(p.x, 0) - c[0], coord(p.y, 1) - c[1], coord(p.z, 2) - c[2]);
+                }
+            });
+        },
+        // A child cell is one level below its parent (a cell with one non-empty octant still has that octant
+        // as its child), so its centre is the parent's moved by a quarter of the parent's side along each
+        // axis, in the direction its octal digit gives: a power of two, exact in float.
+        [&](int c, int lev) -> unsigned {
+            return rel && c >= 0 ? (unsigned)(keys[L.nI[c].z] >> (3 * (EVOL_MAXLEVEL - lev))) & 7u : 0u;
+        },
+        [&](int id, const int4 &I, int c, unsigned digit) {
+            T ms[4] = {0, 0, 0, 0}, cc[3] = {0, 0, 0}, cq[6] = {0, 0, 0, 0, 0, 0}, M = 0;
+            float bx[8];
+            box(bx);
+            if (c >= 0) {
+                const float4 bl = __ldcg(&o.bmin[c]), bh = __ldcg(&o.bmax[c]);
+                if (rel) {
+                    const float4 co = __ldcg(&o.coff[c]), Q0 = __ldcg(&o.nQ0[c]), Q1 = __ldcg(&o.nQ1[c]);
+                    const float q = ldexpf(fcube[4 * sys_sorted[I.z] + 3], -(I.x & 0xff) - 2);
+                    M = (T)co.w;
+                    cc[0] = (T)co.x + (T)((digit & 4u) ? q : -q);
+                    cc[1] = (T)co.y + (T)((digit & 2u) ? q : -q);
+                    cc[2] = (T)co.z + (T)((digit & 1u) ? q : -q);
+                    cq[0] = (T)Q0.x; cq[1] = (T)Q0.y; cq[2] = (T)Q0.z;
+                    cq[3] = (T)Q1.x; cq[4] = (T)Q1.y; cq[5] = (T)Q1.z;
+                } else {
+                    M = (T)__ldcg(&o.M64[c]);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) cc[a] = (T)__ldcg(&o.C64[3 * (size_t)c + a]);
+#pragma unroll
+                    for (int a = 0; a < 6; ++a) cq[a] = (T)__ldcg(&o.Q64[6 * (size_t)c + a]);
+                }
+                ms[0] = M;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) ms[1 + a] = M * cc[a];
+                bx[0] = bl.x; bx[1] = bl.y; bx[2] = bl.z;
+                bx[3] = -bh.x; bx[4] = -bh.y; bx[5] = -bh.z;
+                bx[6] = -bl.w;
+            }
+            finish(id, I.x & 0xff, I.z, ms, bx, [&](const T (&cm)[3], T (&q)[8]) {
+                if (c >= 0) {
+#pragma unroll
+                    for (int a = 0; a < 6; ++a) q[a] = cq[a];
+                    quad(q, M, cc[0] - cm[0], cc[1] - cm[1], cc[2] - cm[2]);
+                }
+            });
+        });
+}
+
+// What a node's users need beside its moments, one thread per node: the centre of mass and squared opening
+// radius, centre and half widths of the box, the distance between the centres of mass and cell.
+__global__ void k_node_geometry(const int32_t *__restrict__ nnodes, const int4 *__restrict__ nI,
+                                const uint64_t *__restrict__ keys, const double *__restrict__ cube,
+                                const float *__restrict__ fcube, const int32_t *__restrict__ sys_sorted, float theta,
+                                NodeOut o, int mixed)
+{
+    const int nn = *nnodes;
+    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nn; id += gridDim.x * blockDim.x) {
+        const int4 I = nI[id];
+        const int lev = I.x & 0xff, sys = sys_sorted[I.z];
+        const uint64_t key0 = keys[I.z];
+        const float4 lo = o.bmin[id], hi = o.bmax[id];
+        float com[3], delta;
+        if (mixed) {
+            double dd = 0.0;
+            const double side = ldexp(cube[4 * sys + 3], -lev);
+            for (int a = 0; a < 3; ++a) {
+                const double c = o.C64[3 * (size_t)id + a];
+                const double off = c - (cube[4 * sys + a] + ((double)cell_index(key0, lev, a) + 0.5) * side);
+                com[a] = (float)c;
+                dd += off * off;
+            }
+            delta = (float)sqrt(dd);
+        } else {
+            const float4 co = o.coff[id];
+            const float off[3] = {co.x, co.y, co.z};
+            float s = 0.f, err = 0.f;              // sum of squares s + err, its error far below FP32's
+            for (int a = 0; a < 3; ++a) {
+                const Centre cg = node_centre(fcube[4 * sys + a], fcube[4 * sys + 3], cell_index(key0, lev, a), lev);
+                const Centre t = two_sum(cg.hi, off[a]);
+                com[a] = t.hi + (t.lo + cg.lo);
+                const float sq = __fmul_rn(off[a], off[a]);
+                const Centre u = two_sum(s, sq);
+                s = u.hi;
+                err += u.lo + fmaf(off[a], off[a], -sq);
+            }
+            delta = sqrtf(s);
+            if (delta > 0.f && delta < 1e18f) delta += __fdividef(0.5f * (fmaf(-delta, delta, s) + err), delta);
+        }
+        const float l = ldexpf(fcube[4 * sys + 3], -lev);
+        const float ropen = theta > 0.f ? l / theta + delta : INFINITY;
+        o.nA[id] = make_float4(com[0], com[1], com[2], ropen * ropen);
+        o.nB[id] = make_float4(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z), lo.w != 0.f ? 0.f : -1.f);
+        o.nC[id] = make_float4(0.5f * (hi.x - lo.x), 0.5f * (hi.y - lo.y), 0.5f * (hi.z - lo.z), 0.f);
+        reinterpret_cast<float *>(o.nQ1)[4 * (size_t)id + 3] = delta;
     }
 }
 
 // Node maxima of 2 eps (all particles) and 2 h (gas), leaf-up like the moments.
-__device__ __forceinline__ void leaf_len(int b, int e, int n_gas, const int32_t *__restrict__ orig,
-                                         const float *__restrict__ le, const float *__restrict__ lh, float &em,
-                                         float &hm)
+__global__ void __launch_bounds__(128, 8)
+    k_node_lengths(Links L, int n_gas, const int32_t *__restrict__ orig, const float *__restrict__ le,
+                   const float *__restrict__ lh, float4 *nB, float4 *nC)
 {
-    em = 0.f;
-    hm = -1.f;
-    for (int s = b; s < e; ++s) {
-        em = fmaxf(em, le[s]);
-        if (orig[s] < n_gas) hm = fmaxf(hm, lh[s]);
-    }
-}
-
-__global__ void k_node_lengths(const int32_t *__restrict__ nnodes, int n_gas, const int32_t *__restrict__ nbeg,
-                               const int32_t *__restrict__ nend, const int32_t *__restrict__ nnext,
-                               const int32_t *__restrict__ nparent, const int32_t *__restrict__ nnch,
-                               int32_t *__restrict__ narrive, const int32_t *__restrict__ orig,
-                               const float *__restrict__ le, const float *__restrict__ lh, float4 *nB, float4 *nC,
-                               int *err)
-{
-    int nn = *nnodes;
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nn; id += gridDim.x * blockDim.x) {
-        if (nnch[id] != 0) continue;
-        float em, hm;
-        leaf_len(nbeg[id], nend[id], n_gas, orig, le, lh, em, hm);
-        nC[id].w = 2.f * em;
-        nB[id].w = hm >= 0.f ? 2.f * hm : -1.f;
-        __threadfence();
-        int p = nparent[id];
-        for (int climb = 0; p >= 0 && p < nn; ++climb) {
-            if (climb > EVOL_MAXLEVEL + 1) {     // deeper than the tree can be: corrupt parents
-                evol_flag(err, EVOL_ETIMEOUT);
-                break;
-            }
-            int old = atomicAdd(&narrive[p], 1);
-            if (old != nnch[p] - 1) break;
-            __threadfence();
-            float e2 = 0.f, h2 = -1.f;
-            for (int c = p + 1; c < nn && __ldcg(&nbeg[c]) < nend[p]; c = __ldcg(&nnext[c])) {
-                e2 = fmaxf(e2, __ldcg(&nC[c].w));
-                h2 = fmaxf(h2, __ldcg(&nB[c].w));
-            }
-            nC[p].w = e2;
-            nB[p].w = h2;
-            __threadfence();
-            p = nparent[p];
+    const int sub = threadIdx.x & 7;
+    auto finish = [&](int id, float em, float hm) {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            em = fmaxf(em, __shfl_xor_sync(0xffffffffu, em, o));
+            hm = fmaxf(hm, __shfl_xor_sync(0xffffffffu, hm, o));
         }
-    }
+        if (id >= 0 && sub == 0) nC[id].w = em;
+        if (id >= 0 && sub == 1) nB[id].w = hm >= 0.f ? hm : -1.f;
+    };
+    leaf_up(
+        L,
+        [&](int id, const int4 &I) {
+            float em = 0.f, hm = -1.f;
+            for (int s = I.z + sub; id >= 0 && s < I.w; s += 8) {
+                em = fmaxf(em, 2.f * le[s]);
+                if (orig[s] < n_gas) hm = fmaxf(hm, 2.f * lh[s]);
+            }
+            finish(id, em, hm);
+        },
+        [](int, int) { return 0; },
+        [&](int id, const int4 &, int c, int) {
+            finish(id, c >= 0 ? __ldcg(&nC[c].w) : 0.f, c >= 0 ? __ldcg(&nB[c].w) : -1.f);
+        });
 }
 
 // ---- several independent systems (batched): per-system cube and keys ----------------------
@@ -986,12 +1093,6 @@ __global__ void k_keys_sorted(int n, const float *__restrict__ x, const float *_
     const int sy = sys_of_pos(sys_off, nsys, j);
     keys[s] = key_of(x[j], y[j], z[j], cube + 4 * sy);
     if (vals_out) vals_out[s] = j;
-}
-
-__global__ void k_zero_i32(const int32_t *__restrict__ nnodes, int32_t *a)
-{
-    int nn = *nnodes;
-    for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < nn; id += gridDim.x * blockDim.x) a[id] = 0;
 }
 
 }  // namespace
@@ -1125,25 +1226,19 @@ int evol_launch_build(evol_ctx *c, const evol_particles *p, const evol_params *p
     k_link<<<ng, 256, 0, st>>>(d.nnodes, leaf, d.nbeg, d.nend, d.nlev, d.nnext, d.nparent, d.nnch, d.narrive, d.nI,
                                d.nK0, d.nK1, nsys, d.sys_off, d.base, d.sys_root);
     NodeOut o{d.nA, d.nB, d.nC, d.nQ0, d.nQ1, d.nBmin, d.nBmax, d.nCoff, d.nM64, d.nC64, d.nQ64};
-    float theta = prm->theta;
-    if (prm->precision == EVOL_FP32_MIXED)
-        k_moments<double><<<ng, 128, 0, st>>>(d.nnodes, (int)p->n_gas, d.nbeg, d.nend, d.nlev, d.nnext, d.nparent,
-                                              d.nnch, d.narrive, d.pos, d.orig, d.keys_a, d.cube, d.sys_sorted, theta,
-                                              o, 1, d.err);
-    else
-        k_moments<float><<<ng, 128, 0, st>>>(d.nnodes, (int)p->n_gas, d.nbeg, d.nend, d.nlev, d.nnext, d.nparent,
-                                             d.nnch, d.narrive, d.pos, d.orig, d.keys_a, d.cube, d.sys_sorted, theta,
-                                             o, 0, d.err);
+    const Links L{d.nnodes, d.nparent, d.nnch, d.nI, d.nK0, d.nK1, d.narrive, d.err};
+    const bool mixed = prm->precision == EVOL_FP32_MIXED;
+    if (mixed) k_moments<double><<<c->num_sms * 5, 128, 0, st>>>(L, (int)p->n_gas, d.pos, d.orig, d.keys_a, d.fcube, d.sys_sorted, o);
+    else k_moments<float><<<c->num_sms * 8, 128, 0, st>>>(L, (int)p->n_gas, d.pos, d.orig, d.keys_a, d.fcube, d.sys_sorted, o);
+    k_node_geometry<<<ng, 256, 0, st>>>(d.nnodes, d.nI, d.keys_a, d.cube, d.fcube, d.sys_sorted, prm->theta, o, mixed);
     return evol_cuda_ok(cudaGetLastError());
 }
 
 int evol_launch_node_lengths(evol_ctx *c, const evol_params *prm, int n_gas)
 {
     evol_dev &d = c->d;
-    int ng = c->num_sms * 8;
     (void)prm;
-    k_zero_i32<<<ng, 256, 0, c->stream>>>(d.nnodes, d.narrive);
-    k_node_lengths<<<ng, 128, 0, c->stream>>>(d.nnodes, n_gas, d.nbeg, d.nend, d.nnext, d.nparent,
-                                              d.nnch, d.narrive, d.orig, d.len_eps, d.len_h, d.nB, d.nC, d.err);
+    const Links L{d.nnodes, d.nparent, d.nnch, d.nI, d.nK0, d.nK1, d.narrive, d.err};
+    k_node_lengths<<<c->num_sms * 8, 128, 0, c->stream>>>(L, n_gas, d.orig, d.len_eps, d.len_h, d.nB, d.nC);
     return evol_cuda_ok(cudaGetLastError());
 }
