@@ -164,6 +164,43 @@ __device__ __forceinline__ double key_scale(double side)
     return ldexp(1.0, EVOL_MAXLEVEL + 1 - e);
 }
 
+// The sum of two floats as a float and what its rounding left out, exactly.
+struct Centre {
+    float hi, lo;
+};
+
+__device__ __forceinline__ Centre two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+
+// One axis' cell, floor((x - corner) 2^21 / side) of the difference rounded to double, in float arithmetic (FP64
+// units made the key kernel ten times as long as its reads and writes: 3.1 M particles 161 -> 60 us).  x - corner
+// is d.hi + d.lo exactly and the scale a power of two, so the floor is that of d.hi unless d.hi falls on a
+// cell's edge and d.lo lies below it; a d.lo that double would have rounded away is left to double.
+__device__ __forceinline__ uint64_t axis_cell(float x, double corner, float scale, double side)
+{
+    const Centre d = two_sum(x, -(float)corner);
+    const float t = d.hi * scale;
+    float q = floorf(t);
+    const float lim = d.hi * 0x1p-52f;
+    const bool edge = q == t && d.lo < 0.f;
+    if (edge) q -= 1.f;
+    if (scale == 0.f || (edge && !(lim >= 0x1p-126f && -d.lo > lim)))
+        q = (float)fmin(fmax(floor(__dmul_rn(__dsub_rn((double)x, corner), key_scale(side))), 0.0), 2097151.0);
+    return (uint64_t)fminf(fmaxf(q, 0.f), 2097151.f);
+}
+
+__device__ __forceinline__ uint64_t key_of(float x, float y, float z, const double *__restrict__ cb)
+{
+    // 2^21 / side where it is a normal float, else 0
+    const int e = ilogb(cb[3]);
+    const float scale = e > -100 && e < 126 ? __int_as_float((127 + EVOL_MAXLEVEL - e) << 23) : 0.f;
+    return (spread3(axis_cell(x, cb[0], scale, cb[3])) << 2) | (spread3(axis_cell(y, cb[1], scale, cb[3])) << 1) |
+           spread3(axis_cell(z, cb[2], scale, cb[3]));
+}
+
 // hist, if given, counts the first digit of the radix sort per tile (zeroed by the caller).
 __global__ void k_keys(int n, const float *__restrict__ x, const float *__restrict__ y, const float *__restrict__ z,
                        const double *__restrict__ cube, uint64_t *__restrict__ keys, int32_t *__restrict__ vals,
@@ -171,17 +208,7 @@ __global__ void k_keys(int n, const float *__restrict__ x, const float *__restri
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double scale = key_scale(cube[3]);
-    float v[3] = {x[i], y[i], z[i]};
-    uint64_t q[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        double s = floor(__dmul_rn(__dsub_rn((double)v[a], cube[a]), scale));
-        s = s < 0.0 ? 0.0 : s;
-        s = s > 2097151.0 ? 2097151.0 : s;
-        q[a] = (uint64_t)s;
-    }
-    const uint64_t key = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
+    const uint64_t key = key_of(x[i], y[i], z[i], cube);
     keys[i] = key;
     vals[i] = i;
     if (hist) atomicAdd(&hist[(i / RS_TILE) * 256 + (int)(key & 255u)], 1);
@@ -573,9 +600,7 @@ __global__ void k_fill(int n, const uint64_t *__restrict__ keys, const int8_t *_
         if (total > node_cap) evol_flag(err, EVOL_EOVERFLOW);
     }
     if (i >= n) return;
-    int lo;
-    int c = nodes_at(n, lcp, i, leaf, lo);
-    int b = base[i];
+    const int lo = lcp[i] + 1, b = base[i], c = base[i + 1] - b;
     const int send = sys_off[sys_sorted[i] + 1];
     for (int k = 0; k < c; ++k) {
         int id = b + k;
@@ -658,16 +683,6 @@ __device__ __forceinline__ unsigned cell_index(uint64_t key0, int lev, int a)
 // A node's geometric centre along one axis, as the sum of two floats.  The cube's corner is a float, and the
 // centre's offset from it an odd number of 22 bits times a power of two, so the sum of the two in hi + lo is
 // exact, and a float minus the centre is right to the rounding of the result, without double arithmetic.
-struct Centre {
-    float hi, lo;
-};
-
-__device__ __forceinline__ Centre two_sum(float a, float b)
-{
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-
 __device__ __forceinline__ Centre node_centre(float corner, float side, unsigned cell, int lev)
 {
     return two_sum(corner, (float)(2u * cell + 1u) * ldexpf(side, -lev - 1));
@@ -1039,20 +1054,6 @@ __global__ void k_bbox_sys(int n, int32_t *__restrict__ sys_off, const float *__
             sys_off[1] = n;
         }
     }
-}
-
-__device__ __forceinline__ uint64_t key_of(float x, float y, float z, const double *__restrict__ cb)
-{
-    const double scale = key_scale(cb[3]);
-    const float v[3] = {x, y, z};
-    uint64_t q[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        double t = floor(__dmul_rn(__dsub_rn((double)v[a], cb[a]), scale));
-        t = t < 0.0 ? 0.0 : (t > 2097151.0 ? 2097151.0 : t);
-        q[a] = (uint64_t)t;
-    }
-    return (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
 }
 
 // keys in the caller's order, each relative to its own system's cube

@@ -32,14 +32,14 @@ def _positions(n, cells, seed):
     return (r.normal(size=(n, 3)) * np.array([1.0, 0.3, 1e-3]) + np.array([3.0, -1e-3, 40.0])).astype(np.float32)
 
 
-def _check(offs, cells, seed):
+def _check(offs, cells, seed, x=None):
     import torch
     from paper_0912_1786_gb300 import build, evol as E
     from paper_0912_1786_gb300.device import DeviceSet
 
     build.build()
     n = offs[-1]
-    x = np.concatenate([_positions(b - a, cells, seed + k) for k, (a, b) in enumerate(zip(offs[:-1], offs[1:]))])
+    x = x if x is not None else np.concatenate([_positions(b - a, cells, seed + k) for k, (a, b) in enumerate(zip(offs[:-1], offs[1:]))])
     zero = np.zeros(n, np.float32)
     one = np.ones(n, np.float32)
     w = W.Workload("sort", x=x[:, 0].copy(), y=x[:, 1].copy(), z=x[:, 2].copy(), vx=zero, vy=zero, vz=zero, m=one,
@@ -76,3 +76,20 @@ def test_several_systems(systems, size, cells):
     # sizes differ: every third system is a single particle
     sizes = [1 if k % 3 == 2 else size + k % 5 for k in range(systems)]
     _check([0] + [int(v) for v in np.cumsum(sizes)], cells, systems)
+
+
+@pytest.mark.parametrize("low", [0.0, 1e-9, -1e-9, 1e-25, -1e-25, 1e-43, 0.3, -7.7, 1e6])
+@pytest.mark.parametrize("size", [1.0, 3.7e-6, 2.5e9, 1e-36, 1e30])
+def test_cell_edges(low, size):
+    # positions on and next to the edges of cells, with corners that the differences to them round away in
+    # float, in double, or not at all: the keys are formed in float arithmetic but must be those of double
+    r = np.random.default_rng(int(abs(np.log(size)) * 10))
+    lo = np.float32(low)
+    t = (r.integers(0, 2 ** 21, (4000, 3)) / 2.0 ** 21 * size).astype(np.float32)
+    t[:1500] += lo                                             # edges counted from the corner
+    step = r.integers(-1, 2, t.shape)
+    x = np.where(step > 0, np.nextafter(t, np.float32(np.inf)), np.where(step < 0, np.nextafter(t, lo), t))
+    x = np.maximum(x, lo).astype(np.float32)
+    x[0] = lo
+    x[1] = lo + np.float32(size)
+    _check([0, len(x)], 0, 0, x)
