@@ -41,8 +41,8 @@ FLOPS_PP_NEWTON = 19
 FLOPS_PP_SOFT = 89
 FLOPS_SPH = 85
 # Algorithmic DRAM bytes per particle of the tree build (one pass over each kernel's inputs and
-# outputs): bbox 12, keys 12 + 12, 8 radix passes x (histogram 8 + scatter 24), permute 40 + 44,
-# common prefixes 8 + 5, node counts 5, their scan 16, moments 20; plus per node: fill 16,
+# outputs): bbox 12, keys 12 + 12, 8 radix passes x (histogram 8 + scatter 24), permute 40 + 44
+# and common prefixes 8 + 5, node counts 5, their scan 16, moments 20; plus per node: fill 16,
 # link 80, moments 150.
 BUILD_BYTES_PER_PARTICLE = 12 + 24 + 8 * 32 + 84 + 13 + 5 + 16 + 20
 BUILD_BYTES_PER_NODE = 16 + 80 + 150
@@ -869,15 +869,31 @@ def main():
 
 
 def launches_per_step(w):
-    """Kernels of ours per evol_step: bbox 2, keys 1, 8 radix passes x (hist + 3 scan + scatter),
-    permute, lcp, count, 3 scan, fill, link, moments, eps solve, h solve, pack, node-lengths 2,
-    walk, unpermute, diagnostics 2."""
-    p = w.params
-    k = 2 + 1 + 8 * 5 + 1 + 1 + 1 + 3 + 1 + 1 + 1
-    k += 1 if (p.gravity and p.adaptive_softening) else 0
-    k += 1 if (p.sph and w.n_gas) else 0
-    k += 1 + 2 + 1 + 1 + 2
-    return k
+    """Kernels of ours per evol_step (the device chooses nothing here: both block shapes of a length
+    solve and both forms of a split walk are launched, one returns at once)."""
+    p, n = w.params, w.n
+    nsys = 1 if w.sys_offsets is None else len(w.sys_offsets) - 1
+    scan = lambda m: 1 if m <= 16384 else 3
+    digits = 1 if nsys > 1 else 0
+    while nsys > 256 ** digits and nsys > 1:
+        digits += 1
+    k = (1 if n <= 12288 or nsys > 1 else 2) + 1                       # bounding cube, keys
+    if n <= 12288:
+        k += 1                                                         # direct ranking
+    else:
+        one = 1 if n <= 131072 else 2 + scan(256 * ((n + 2047) // 2048))
+        k += (8 + digits) * one + (2 if nsys > 1 else 0)               # passes; systems: ids, keys again
+    k += 1 + 1 + scan(n) + 1 + 1 + 2                                   # permute, counts, nodes, links, moments
+    eps, h = bool(p.gravity and p.adaptive_softening), bool(p.sph and w.n_gas)
+    shared = eps and h and w.n_gas == n and p.n_nei_grav == p.n_nei_sph
+    if h and w.n_gas < n:
+        k += 2 + scan(n)                                               # gas lists
+    k += (int(eps) + int(h) - int(shared)) * (3 if n >= 65536 else 1)  # leaf lists and two shapes
+    k += 1 + 1                                                         # operands, node lengths
+    ewald = p.gravity and p.periodic_mask
+    k += 0 if ewald else 1                                             # super-groups
+    k += 3 if (n <= 58368 and not ewald) else 1                        # walk
+    return k + 1 + 2                                                   # results, diagnostics
 
 
 def replica_rate(dist, device, ms_local, units_per_rank, steps, world):

@@ -337,6 +337,8 @@ int evol_get_diagnostics(evol_ctx *ctx, double out[16]);
  *        candidates, [+1] gathers by a particle's own tree walk, [+2] neighbour lists that overflowed,
  *        [+3] times a block's candidates did not fit
  *   [24] eps-solve and [25] h-solve Newton iterations (sum over particles)
+ *   Where h and eps solve the same equation (all gas, equal neighbour numbers) one solve serves both
+ *   and counts as both; [3] counts it once.
  *   [26..31] zero */
 int evol_get_counters(evol_ctx *ctx, uint64_t out[32]);
 
@@ -383,8 +385,9 @@ int evol_set_check_mode(evol_ctx *ctx, int on);
  * that path.  Takes effect from the next call.  Returns EVOL_EINVAL out of range. */
 int evol_set_stack_limit(evol_ctx *ctx, int64_t entries);
 
-/* Event timings (ms) of the phases of the last evol_step: [0] build, [1] eps solve,
- * [2] h solve, [3] force walk, [4] total. Valid after evol_sync. */
+/* Event timings (ms) of the phases of the last evol_step: [0] build, [1] eps solve (or the one
+ * solve for h and eps), [2] h solve (if it is one of its own), node maxima of the lengths and operands of the
+ * walk, [3] force walk, [4] total. Valid after evol_sync. */
 int evol_get_timings(evol_ctx *ctx, float out[5]);
 
 /* Allocation-free key + sort stage (the paper has no counterpart: this is a service for callers

@@ -323,7 +323,7 @@ int evol_create(evol_ctx **out, int64_t max_n, void *stream)
         rc |= dalloc(&d.wpart, (16 * ngr < most ? 16 * ngr : most) * EVOL_PART_FLOATS);
     }
     rc |= dalloc(&d.nbmin, n); rc |= dalloc(&d.bt, 8);
-    rc |= dalloc(&d.ewald, (int64_t)EVOL_EWALD_M * EVOL_EWALD_M * EVOL_EWALD_M);
+    rc |= dalloc(&d.ewald, (int64_t)EVOL_EWALD_M * EVOL_EWALD_M * EVOL_EWALD_N * 2);
     if (!rc && cudaMallocHost((void **)&c->h_bt, 8 * sizeof(unsigned long long)) != cudaSuccess) rc = EVOL_ENOMEM;
     rc |= dalloc(&d.dt, 4); rc |= dalloc(&d.time, 1);
     rc |= dalloc(&d.keys_a, n); rc |= dalloc(&d.keys_b, n); rc |= dalloc(&d.vals_a, n); rc |= dalloc(&d.vals_b, n);

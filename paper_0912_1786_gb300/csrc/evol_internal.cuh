@@ -61,7 +61,8 @@ struct evol_dev {
     unsigned long long *sg_stat;     // and the candidates of all super-groups, and their number
     unsigned *nbmin;                // sorted: smallest active-neighbour step (wake-up)
     unsigned long long *bt;         // [0] t_sys [1] t_next (ticks); [2..5] run counts
-    float4 *ewald;                  // periodic gravity: correction table (f, g) for L = 1
+    float4 *ewald;                  // periodic gravity: correction table (f, g) for L = 1, each
+                                    // point beside either neighbour in z
     float *dt;               // integrator scalars: [0] time step, [1] criterion minimum (as bits)
     double *time;            // integrator time
     float *dudt;             // sorted

@@ -754,12 +754,18 @@ __global__ void k_ewald_table(float4 *tab)
             }
     g += pi / (w * w);
     const float f0 = (float)F[0], f1 = (float)F[1], f2 = (float)F[2], fg = (float)g;
-    tab[(i * M + j) * M + k] = make_float4(f0, f1, f2, fg);
-    tab[(i * M + k) * M + j] = make_float4(f0, f2, f1, fg);
-    tab[(j * M + i) * M + k] = make_float4(f1, f0, f2, fg);
-    tab[(j * M + k) * M + i] = make_float4(f1, f2, f0, fg);
-    tab[(k * M + i) * M + j] = make_float4(f2, f0, f1, fg);
-    tab[(k * M + j) * M + i] = make_float4(f2, f1, f0, fg);
+    // each point beside both its neighbours along the last axis
+    auto put = [&](int a, int b, int c, float fa, float fb, float fc) {
+        float4 *row = tab + 2 * ((a * M + b) * N);
+        if (c < N) row[2 * c] = make_float4(fa, fb, fc, fg);
+        if (c > 0) row[2 * c - 1] = make_float4(fa, fb, fc, fg);
+    };
+    put(i, j, k, f0, f1, f2);
+    put(i, k, j, f0, f2, f1);
+    put(j, i, k, f1, f0, f2);
+    put(j, k, i, f1, f2, f0);
+    put(k, i, j, f2, f0, f1);
+    put(k, j, i, f2, f1, f0);
 }
 
 }  // namespace

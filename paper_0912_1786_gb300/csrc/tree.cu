@@ -1,5 +1,5 @@
-// Tree build on the GPU (Sect. 2.2 of the paper): root cube, 63-bit Morton keys, stable LSD
-// radix sort, particle permutation, pre-order octree from the sorted keys, and node moments
+// Tree build on the GPU (Sect. 2.2 of the paper): root cube, 63-bit Morton keys, stable sort,
+// particle permutation, pre-order octree from the sorted keys, and node moments
 // reduced bottom-up.
 //
 // Node construction does not insert particles one by one.  With keys sorted, the cells of

@@ -154,10 +154,17 @@ __device__ __forceinline__ int nth_bit(unsigned m, int k)
 // Periodic gravity: trilinear interpolation in the Ewald table (Sect. 4.3).  f is odd in its own
 // coordinate and even in the others, g is even, so the table holds the octant [0, L/2]^3 only; the
 // four components are interpolated as two packed pairs, (f_x, f_y) and (f_z, g), and the caller
-// applies the octant signs.  sc = 2 N / L.
+// applies the octant signs.  sc = 2 N / L.  The periodic walk is bound by the L1 wavefronts of these loads, one for
+// nearly every lane and load, so a point is stored twice, beside either neighbour in z, and a lookup is four
+// loads of 32 bytes: 7.04 -> 6.68 ms for 262 k particles against eight of 16.
 struct Ew2 {
     f32x2 xy, zw;
 };
+// Two neighbouring points of the table, which holds them side by side, in one 32-byte load.
+__device__ __forceinline__ void load_pair(const float4 *p, ulonglong2 &a, ulonglong2 &b)
+{
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(a.x), "=l"(a.y), "=l"(b.x), "=l"(b.y) : "l"(p));
+}
 __device__ __forceinline__ Ew2 ewald_lookup2(const float4 *__restrict__ tab, float dx, float dy, float dz, float sc)
 {
     const int M = EVOL_EWALD_M;
@@ -167,9 +174,13 @@ __device__ __forceinline__ Ew2 ewald_lookup2(const float4 *__restrict__ tab, flo
     // every index stays inside the table; truncation is the floor for the non-negative values
     const int i = __float2int_rz(fminf(ux, nm1)), j = __float2int_rz(fminf(uy, nm1)), k = __float2int_rz(fminf(uz, nm1));
     const float tx = ux - (float)i, ty = uy - (float)j, tz = uz - (float)k;
-    const ulonglong2 *b = reinterpret_cast<const ulonglong2 *>(tab + ((i * M + j) * M + k));
-    const ulonglong2 c000 = b[0], c001 = b[1], c010 = b[M], c011 = b[M + 1];
-    const ulonglong2 c100 = b[M * M], c101 = b[M * M + 1], c110 = b[M * M + M], c111 = b[M * M + M + 1];
+    const float4 *b = tab + 2 * ((i * M + j) * EVOL_EWALD_N + k);
+    constexpr int J = 2 * EVOL_EWALD_N, I = M * J;
+    ulonglong2 c000, c001, c010, c011, c100, c101, c110, c111;
+    load_pair(b, c000, c001);
+    load_pair(b + J, c010, c011);
+    load_pair(b + I, c100, c101);
+    load_pair(b + I + J, c110, c111);
     const f32x2 TZ = pk2(tz, tz), TY = pk2(ty, ty), TX = pk2(tx, tx);
     auto L = [](f32x2 a, f32x2 c, f32x2 t) { return fma2(t, sub2(c, a), a); };
     const f32x2 a0 = L(c000.x, c001.x, TZ), b0 = L(c000.y, c001.y, TZ);
