@@ -149,6 +149,7 @@ struct evol_ctx {
     uint64_t bins_sig;
     unsigned long long *h_bt;        // pinned host copy of the system time
     int ewald_ready;                 // the Ewald table has been computed
+    void *arrays;                    // the allocation that holds every device array
 };
 
 // ---- host-side launch helpers (defined in evol_api.cu / tree.cu / walks) ------------------
