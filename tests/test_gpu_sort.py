@@ -71,7 +71,7 @@ def test_one_system(n, cells):
 
 
 @pytest.mark.parametrize("cells", [0, 4])
-@pytest.mark.parametrize("systems,size", [(2, 33), (300, 37), (300, 50), (257, 509), (700, 200)])
+@pytest.mark.parametrize("systems,size", [(2, 33), (300, 37), (300, 50), (257, 509), (700, 200), (3, 2999), (3, 9000)])
 def test_several_systems(systems, size, cells):
     # sizes differ: every third system is a single particle
     sizes = [1 if k % 3 == 2 else size + k % 5 for k in range(systems)]
