@@ -805,10 +805,23 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 5)
 {
     constexpr bool rel = sizeof(T) == sizeof(float);
     const int lane = threadIdx.x & 31, sub = lane & 7, oct = lane & 24;
-    // an octet's node from its lanes' shares: mass and mass times position, box (lo, -hi, -gas), then the
-    // quadrupole shares that add_q makes about the centre of mass
+    // Adds the lanes' masses and masses times positions to the octet's sums.  FP32: one after the other in
+    // the order of the particles or children, on every lane, so that a node's opening radius, on which the walk's
+    // decisions turn, does not depend on how the lanes split it; FP64: each lane its own, summed by finish.
+    auto add = [&](T (&ms)[4], T w, T x, T y, T z) {
+#pragma unroll
+        for (int k = 0; k < (rel ? 8 : 1); ++k) {
+            const T wk = rel ? __shfl_sync(0xffffffffu, w, oct + k) : w;
+            ms[0] += wk;
+            ms[1] += wk * (rel ? __shfl_sync(0xffffffffu, x, oct + k) : x);
+            ms[2] += wk * (rel ? __shfl_sync(0xffffffffu, y, oct + k) : y);
+            ms[3] += wk * (rel ? __shfl_sync(0xffffffffu, z, oct + k) : z);
+        }
+    };
+    // an octet's node from its sums and its lanes' shares: box (lo, -hi, -gas), then the quadrupole shares that
+    // add_q makes about the centre of mass
     auto finish = [&](int id, int lev, int beg, T (&ms)[4], float (&bx)[8], auto add_q) {
-        const T sum = octet_sum4(ms, sub);
+        const T sum = rel ? (sub == 0 ? ms[0] : sub == 1 ? ms[1] : sub == 2 ? ms[2] : ms[3]) : octet_sum4(ms, sub);
         const float bound = octet_reduce(bx, sub, [](float a, float b) { return fminf(a, b); });
         const T M = __shfl_sync(0xffffffffu, sum, oct);
         T c[3];
@@ -882,14 +895,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 5)
             T ms[4] = {0, 0, 0, 0};
             float bx[8];
             box(bx);
-            for (int s = b + sub; s < e; s += 8) {
-                const float4 p = pos[s];
+            for (int s = b + sub; __any_sync(0xffffffffu, s < e); s += 8) {
+                const bool in = s < e;
+                const float4 p = in ? pos[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+                add(ms, (T)p.w, in ? coord(p.x, 0) : (T)0, in ? coord(p.y, 1) : (T)0, in ? coord(p.z, 2) : (T)0);
+                if (!in) continue;
                 if (orig[s] < n_gas) bx[6] = -1.f;
-                const T w = (T)p.w;
-                ms[0] += w;
-                ms[1] += w * coord(p.x, 0);
-                ms[2] += w * coord(p.y, 1);
-                ms[3] += w * coord(p.z, 2);
                 bx[0] = fminf(bx[0], p.x); bx[1] = fminf(bx[1], p.y); bx[2] = fminf(bx[2], p.z);
                 bx[3] = fminf(bx[3], -p.x); bx[4] = fminf(bx[4], -p.y); bx[5] = fminf(bx[5], -p.z);
             }
@@ -928,13 +939,11 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 5)
 #pragma unroll
                     for (int a = 0; a < 6; ++a) cq[a] = (T)__ldcg(&o.Q64[6 * (size_t)c + a]);
                 }
-                ms[0] = M;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) ms[1 + a] = M * cc[a];
                 bx[0] = bl.x; bx[1] = bl.y; bx[2] = bl.z;
                 bx[3] = -bh.x; bx[4] = -bh.y; bx[5] = -bh.z;
                 bx[6] = -bl.w;
             }
+            add(ms, M, cc[0], cc[1], cc[2]);
             finish(id, I.x & 0xff, I.z, ms, bx, [&](const T (&cm)[3], T (&q)[8]) {
                 if (c >= 0) {
 #pragma unroll
