@@ -795,8 +795,8 @@ __device__ __forceinline__ void leaf_up(const Links &L, Leaf leaf, Pre pre, Node
 // Moments of every node: mass, centre of mass (FP32: its offset from the node's centre), quadrupole about it, and
 // the particles' box.  Bound by the chain of dependent steps from the leaves to the root, not by its reads.
 // A thread per node, its children one after the other and each in dependent loads, took 54 us with 1000
-// particles, 141 with 49 k and 962 with 3.1 M; this and k_node_geometry take 26, 58 and 274 (FP64 of 393 k:
-// 389 -> 184), k_node_lengths 13, 32 and 154 (26, 77 and 197).
+// particles, 141 with 49 k and 962 with 3.1 M; this and k_node_geometry take 24, 59 and 279 (FP64 of 393 k:
+// 389 -> 184), k_node_lengths 12, 32 and 145 (26, 77 and 197).
 template <typename T>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 5)
     k_moments(Links L, int n_gas, const float4 *__restrict__ pos, const int32_t *__restrict__ orig,
