@@ -313,8 +313,8 @@ __device__ __forceinline__ unsigned long long evol_mix64(unsigned long long z)
     return z ^ (z >> 31);
 }
 
-// Nearest image on an axis of length len (il = 1/len, 0 for an axis that is not periodic): the nearest
-// integer by adding and subtracting 1.5 2^23, exact below 2^22 box lengths.
+// Nearest image on an axis of length len (il = 1/len; both 0 for an axis that is not periodic, where the result
+// is d): the nearest integer by adding and subtracting 1.5 2^23, exact below 2^22 box lengths.
 __device__ __forceinline__ float evol_nearest(float d, float len, float il)
 {
     const float k = (d * il + 12582912.f) - 12582912.f;
@@ -340,7 +340,7 @@ struct evol_kparams {
     float theta, G, gamma, alpha, beta;
     float eta_h, eta_e;
     int gravity, sph, adaptive, use_tc, periodic_mask, mixed;
-    float plen[3], pinv[3];  // periodic lengths; 1/length (0 on an axis that is not periodic)
+    float plen[3], pinv[3];  // periodic lengths and 1/length (both 0 on an axis that is not periodic)
     int n, n_gas, leaf;
     int stack_cap;           // traversal-stack entries a warp may use
     int stack_stride;        // entries allocated per warp (>= stack_cap)
@@ -364,3 +364,14 @@ struct evol_kparams {
     int diss, visc_form, balsara, var_alpha, conduction, cond_vsig, cond_source;
     float alpha_min, alpha_tau, alpha_source, alpha_u_min;
 };
+
+// The periodic lengths of a call.  The bounds of an open axis may hold anything (infinities where it is
+// unbounded, unset values) and are not read.
+static inline void evol_periodic_axes(evol_kparams &kp, const evol_params *prm)
+{
+    for (int a = 0; a < 3; ++a) {
+        const bool periodic = (prm->periodic_mask >> a) & 1;
+        kp.plen[a] = periodic ? prm->periodic_hi[a] - prm->periodic_lo[a] : 0.f;
+        kp.pinv[a] = periodic ? 1.f / kp.plen[a] : 0.f;
+    }
+}

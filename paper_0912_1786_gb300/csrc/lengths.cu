@@ -1374,10 +1374,7 @@ int evol_launch_lengths(evol_ctx *c, const evol_particles *p, const evol_params 
     kp.eta_h = 0.5f * cbrtf(3.f * prm->n_nei_sph / (4.f * EVOL_PI_F));
     kp.eta_e = 0.5f * cbrtf(3.f * prm->n_nei_grav / (4.f * EVOL_PI_F));
     kp.periodic_mask = prm->periodic_mask;
-    for (int a = 0; a < 3; ++a) {
-        kp.plen[a] = prm->periodic_hi[a] - prm->periodic_lo[a];
-        kp.pinv[a] = (prm->periodic_mask >> a) & 1 ? 1.f / kp.plen[a] : 0.f;
-    }
+    evol_periodic_axes(kp, prm);
     kp.active = c->bins_active;
     kp.want_curl = mode != 1 && evol_needs_curl(prm);
     kp.standard = mode == 0 && prm->sph_scheme == EVOL_SPH_STANDARD;

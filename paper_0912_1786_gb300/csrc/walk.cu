@@ -1519,10 +1519,7 @@ int evol_launch_walk(evol_ctx *c, const evol_particles *p, const evol_params *pr
     kp.adaptive = prm->adaptive_softening;
     kp.use_tc = prm->use_tc_gradient;
     kp.periodic_mask = prm->periodic_mask;
-    for (int a = 0; a < 3; ++a) {
-        kp.plen[a] = prm->periodic_hi[a] - prm->periodic_lo[a];
-        kp.pinv[a] = (prm->periodic_mask >> a) & 1 ? 1.f / kp.plen[a] : 0.f;
-    }
+    evol_periodic_axes(kp, prm);
     kp.stack_cap = (int)c->wstack_lim;
     kp.stack_stride = (int)c->wstack_cap;
     kp.active = c->bins_active;
