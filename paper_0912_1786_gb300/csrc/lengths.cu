@@ -198,14 +198,16 @@ __device__ int start_node(const evol_dev &d, const LenSmem<NW, FLOW> &sm, int sy
     for (int q = 0; q < NW; ++q) {
         const float4 G = sm.gc[q], H = sm.gh[q];
         if (G.w < 0.f) continue;
-        // outward by 1e-3 of the radius and a part in 2^20 of the coordinates: far above the rounding here
+        // outward by 1e-3 of the radius and a part in 2^20 of the coordinates, far above the rounding of both, and
+        // by half a finest cell: the offset from the cube's corner is rounded by up to an eighth of one, which is
+        // more than the radius of particles far closer to each other than these cells are wide
         const float R = 1.001f * sqrtf(G.w);
         const float o[3] = {x, y, z}, c[3] = {G.x, G.y, G.z}, h[3] = {H.x, H.y, H.z};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const float r = R + h[a] + 1e-6f * (fabsf(c[a]) + h[a]);
-            const unsigned l = (unsigned)fminf(fmaxf((c[a] - r - o[a]) * sc, 0.f), top);
-            const unsigned u = (unsigned)fminf(fmaxf((c[a] + r - o[a]) * sc, 0.f), top);
+            const unsigned l = (unsigned)fminf(fmaxf((c[a] - r - o[a]) * sc - 0.5f, 0.f), top);
+            const unsigned u = (unsigned)fminf(fmaxf((c[a] + r - o[a]) * sc + 0.5f, 0.f), top);
             if (s0 < 0) c0[a] = l;
             diff |= (l ^ c0[a]) | (u ^ c0[a]);
         }
