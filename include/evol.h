@@ -138,9 +138,10 @@ typedef struct {
     float alpha_u_min;         /* paper: 0 */
     int sph_scheme;            /* EVOL_SPH_LAGRANGIAN (0) or EVOL_SPH_STANDARD; the standard scheme
                                   needs 1 <= n_nei_sph (rounded) <= 335 */
-    int length_group;          /* particles that two warps of the length solves take together (1..32; the
-                                  warps of a block share one list of the leaves near them); 0: chosen
-                                  from the number of particles.  Changes cost, not the definition. */
+    int length_group;          /* length solves: 1..32 sets how many consecutive particles a warp takes -- 1 or
+                                  2 (2 and 3), 4 (4 to 15), 8 (16 and more); the warps of a block share one
+                                  list of the leaves near their particles.  0: chosen from the number of
+                                  particles.  Changes cost, not the definition. */
 } evol_params;
 
 /* Outputs, caller order.  Any pointer may be NULL (not written). */

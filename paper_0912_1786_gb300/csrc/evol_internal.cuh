@@ -355,7 +355,7 @@ struct evol_kparams {
     int part_slots;          // force walk in parts: warps of that variant's grid (0: whole groups only)
     int super;               // the force walk's groups start from their super-group's lists
     int lists;               // the length solves' blocks take their leaves from super-group lists
-    int lsub;                // particles per warp of the length solves (1..32; 0: from their number)
+    int lsub;                // particles per warp of the length solves (1, 2, 4 or 8; 0: from their number)
     // periodic gravity (Ewald): cube side, 2 N / L for the table lookup, the table (L = 1)
     int ewald;
     float ewald_L, ewald_sc;

@@ -1368,6 +1368,14 @@ int launch_lengths_mode(evol_ctx *c, const evol_kparams &kp, unsigned long long 
 
 }  // namespace
 
+// Particles per warp that a caller's length_group stands for (0: group_size chooses): a power of two, so that an
+// item lies inside one quarter of a super-group and can take its leaf list, and at most eight: more of them
+// share a list pass, but their candidates seldom fit a block. eps + h of 2^18 halo + 2^17 gas, ms, with 1, 2,
+// 4, 8 and 16 per warp: 3.07, 2.22, 1.85, 1.84, 2.21; eps of 2^18 Plummer particles 1.36, 0.95, 0.76, 0.75,
+// 0.87. Between, 4 and 8 change places with the set, so 4 is what the sizes up to 15 get (a run of 131 k gas
+// particles 9.83 ms with 4, 9.99 with 8) and 8 is what larger ones ask for.
+static inline int warp_particles(int group) { return group >= 16 ? 8 : group >= 4 ? 4 : group == 3 ? 2 : group; }
+
 int evol_launch_lengths(evol_ctx *c, const evol_particles *p, const evol_params *prm, int mode)
 {
     evol_kparams kp{};
@@ -1382,7 +1390,7 @@ int evol_launch_lengths(evol_ctx *c, const evol_particles *p, const evol_params 
     kp.standard = mode == 0 && prm->sph_scheme == EVOL_SPH_STANDARD;
     kp.nstd = (int)lrintf(prm->n_nei_sph);
     kp.want_divv = c->want_divv || kp.want_curl;
-    kp.lsub = (prm->length_group + 1) / 2;
+    kp.lsub = warp_particles(prm->length_group);
     kp.lists = kp.n >= LISTS_MIN;
     kp.stack_cap = (int)c->wstack_lim;
     kp.stack_stride = (int)c->wstack_cap;

@@ -47,7 +47,7 @@ class Params:
     group_size: int = 32
     use_tc_gradient: int = 1
     sph_scheme: int = 0            # 0: n-h (Lagrangian) scheme; 1: standard scheme, N_nei inside 2h
-    length_group: int = 0          # particles of two warps of the length solves (0: from their number)
+    length_group: int = 0          # sets the particles per warp of the length solves (0: from their number)
     # dissipation variants (Sect. 3.3.3); all off is the standard Monaghan viscosity
     visc_form: int = 0             # 0: Monaghan alpha/beta form; 1: signal-velocity form
     balsara: int = 0               # 1: Balsara limiter on the viscosity
