@@ -68,8 +68,10 @@ constexpr float SEARCH_MARGIN = 1.1f;
 constexpr float NEWTON_TOL = 1e-4f;
 constexpr float CONV_TOL = 1e-6f;
 
-constexpr int LISTS_MIN = 65536;       // below, the blocks' own walks cost less than one more launch (49,152
-                                      // particles: 0.38 ms against 0.41)
+// Particles of a solve (gas of an h solve) from which its leaf lists are made; below, the blocks' own walks cost
+// less than one more launch (h of 20,000 gas particles among 544 k: 0.29 ms against 0.41 with lists, 60,000
+// 0.47 against 0.55; 49,152 of their own 0.38 against 0.41).
+constexpr int LISTS_MIN = 65536;
 constexpr int LEN_SG = 256;           // list entries per super-group of k_leaf_lists (a multiple of 32 per warp)
 constexpr int SG_LEAVES = EVOL_SG_ACAP * LEN_SG / (32 * EVOL_SG_GROUPS);   // leaves of its list at most
 
@@ -1391,7 +1393,7 @@ int evol_launch_lengths(evol_ctx *c, const evol_particles *p, const evol_params 
     kp.nstd = (int)lrintf(prm->n_nei_sph);
     kp.want_divv = c->want_divv || kp.want_curl;
     kp.lsub = warp_particles(prm->length_group);
-    kp.lists = kp.n >= LISTS_MIN;
+    kp.lists = (mode == 0 ? kp.n_gas : kp.n) >= LISTS_MIN;
     kp.stack_cap = (int)c->wstack_lim;
     kp.stack_stride = (int)c->wstack_cap;
     if (mode == 0 && p->n_gas < p->n) {

@@ -91,6 +91,13 @@ def test_every_group_size_takes_the_leaf_lists(group):
     assert items <= g["counters"][5] <= items + blocks
 
 
+@pytest.mark.parametrize("n_gas", [65535, 65536])
+def test_gas_lists_on_both_sides_of_the_line(n_gas):
+    # the leaf lists of an h solve go by the number of gas particles, not by that of all particles
+    w = W.hernquist_gas(20011, n_gas, seed=17)
+    _every_length(w, _step(w), oracle.force_step(w, idx=NONE))
+
+
 @pytest.mark.parametrize("n", [3001, 70001])
 def test_one_solve_for_both_lengths_on_periodic_axes(n):
     w = W.periodic_box(n, seed=8, n_gas=n, sigma_v=0.1)
