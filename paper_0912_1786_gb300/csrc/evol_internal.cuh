@@ -348,6 +348,7 @@ struct evol_kparams {
     int want_divv;           // length solves also form div v
     int want_curl;           // the h solve also forms |curl v| (Balsara limiter, alpha switch)
     int standard, nstd;      // h solve by the standard scheme with nstd neighbours inside 2h
+    int whole;               // length solves: every particle by the whole warp, none four at a time
     // individual time steps: the walks take only the particles of the active list d.act (sorted
     // positions, ascending; its length at d.acts[n]); the force walk also records, per SPH
     // neighbour, the smallest step (ticks) of an active particle next to it (wake-up)

@@ -19,7 +19,8 @@
 //     F = Sw/pi - eta^3,  F' = -Suw/(pi L),  Sw = sum w(u),  Suw = sum u w'(u).
 // Four particles are solved together, eight lanes to each (lists of up to SCAP entries); a particle
 // whose list does not fit, or that fails to converge there, is solved again by the whole warp with a
-// list of up to PCAP entries.
+// list of up to PCAP entries.  Where most lists would not fit (see whole_warp) every particle is
+// solved by the whole warp.
 // Outputs (mode 0, gas h):   rho = Smw/(pi h^3), Omega* = -Suw/(3 Sw),
 //                           zeta = (3 Smw + Smuw)/(3 Sw)          (Sect. 3, Eq. drhodr)
 // Outputs (mode 1, eps):     Upsilon = -Suw/(3 Sw),
@@ -1041,7 +1042,7 @@ __global__ void __launch_bounds__(32 * NW, Shape<NW, FLOW>::MINB) k_lengths(cons
 
             // ---- four particles at a time, eight lanes each, from the staged candidates.  A particle whose
             // radius grows beyond the warp's waits for a later round, which walks for its new length.
-            unsigned solo = (!glist || rounds > MAX_ROUNDS || (MODE == 0 && kp.standard)) ? rm : 0u;
+            unsigned solo = (!glist || rounds > MAX_ROUNDS || kp.whole) ? rm : 0u;
             unsigned fm = rm & ~solo;
             const float *list = nb.r + slot * SCAP;
             while (fm) {
@@ -1378,6 +1379,18 @@ int launch_lengths_mode(evol_ctx *c, const evol_kparams &kp, unsigned long long 
 // particles 9.83 ms with 4, 9.99 with 8) and 8 is what larger ones ask for.
 static inline int warp_particles(int group) { return group >= 16 ? 8 : group >= 4 ? 4 : group == 3 ? 2 : group; }
 
+// Neighbour numbers whose balls (gathered SEARCH_MARGIN wide) mostly leave less than 15 % of a short list free:
+// particles then go to the whole warp and its longer list at once instead of overflowing the short one first.
+// Lengths near their roots, ms, four at a time / whole warp (one warp for each particle and no candidates in
+// shared memory: the form before these): eps of 2^20 Plummer particles inside 4 a, 100 neighbours 4.0 / 4.2
+// (4.5), 130 5.7 / 4.8 (5.7), 160 9.9 / 5.4 (7.1), 200 11.0 / 6.8 (9.6); eps and h of 2^18 halo + 2^17 gas, 80
+// 2.2 / 2.5 (2.6), 110 3.1 / 2.9 (3.3), 130 3.7 / 3.2 (3.9). From poor starting lengths the line lies higher
+// (the halo's 110 4.8 / 6.1, 130 5.9 / 6.7, 160 9.7 / 8.2).
+static inline bool whole_warp(float n_nei)
+{
+    return n_nei * SEARCH_MARGIN * SEARCH_MARGIN * SEARCH_MARGIN > 0.85f * SCAP;
+}
+
 int evol_launch_lengths(evol_ctx *c, const evol_particles *p, const evol_params *prm, int mode)
 {
     evol_kparams kp{};
@@ -1391,6 +1404,7 @@ int evol_launch_lengths(evol_ctx *c, const evol_particles *p, const evol_params 
     kp.want_curl = mode != 1 && evol_needs_curl(prm);
     kp.standard = mode == 0 && prm->sph_scheme == EVOL_SPH_STANDARD;
     kp.nstd = (int)lrintf(prm->n_nei_sph);
+    kp.whole = kp.standard || whole_warp(mode == 0 ? prm->n_nei_sph : prm->n_nei_grav);
     kp.want_divv = c->want_divv || kp.want_curl;
     kp.lsub = warp_particles(prm->length_group);
     kp.lists = (mode == 0 ? kp.n_gas : kp.n) >= LISTS_MIN;

@@ -98,6 +98,30 @@ def test_gas_lists_on_both_sides_of_the_line(n_gas):
     _every_length(w, _step(w), oracle.force_step(w, idx=NONE))
 
 
+def _gas_of_a_halo(n):
+    # h alone: the balls of the halo's outermost particles would hold more than the longest list
+    w = W.hernquist_gas(n, n, seed=9)
+    w.params = dataclasses.replace(w.params, gravity=0, adaptive_softening=0)
+    return w
+
+
+def _with_curl(n):
+    return W.with_dissipation(W.evrard_sphere(n, seed=9), seed=3, sigma_v=0.1, balsara=1)
+
+
+@pytest.mark.parametrize("nnei", [112.0, 113.0, 160.0])
+@pytest.mark.parametrize("make", [lambda: W.evrard_sphere(9001, seed=9), lambda: _gas_of_a_halo(9001), lambda: _with_curl(9001)])
+def test_many_neighbours(make, nnei):
+    # from 113 on particles are solved by whole warps, with lists of twice the length
+    w = make()
+    w.params = dataclasses.replace(w.params, n_nei_sph=nnei, n_nei_grav=nnei)
+    g = _step(w, steps=2)
+    _every_length(w, g, oracle.force_step(w, idx=NONE), ("h", "eps") if w.params.gravity else ("h",))
+    if nnei > 113:
+        # near its root a particle's list is made once, not first a shorter one that overflows
+        assert g["counters"][20] + g["counters"][21] < 1.1 * w.n_gas
+
+
 @pytest.mark.parametrize("n", [3001, 70001])
 def test_one_solve_for_both_lengths_on_periodic_axes(n):
     w = W.periodic_box(n, seed=8, n_gas=n, sigma_v=0.1)
