@@ -840,7 +840,7 @@ def main():
                 "precision": args.precision, "data": "synthetic",
                 "config": {"workload": wname, "n": w.n, "n_gas": w.n_gas, "theta": w.params.theta,
                            "n_nei": w.params.n_nei_sph, "leaf_size": int(ds.params.leaf_size),
-                           "length_group": int(ds.params.length_group) or 8,
+                           "length_group": int(ds.params.length_group),
                            "kdk_steps_per_bench_step": args.kdk_steps or None,
                            "autotune": autotune,
                            "parallelism": "replicas" if world > 1 else "single",
@@ -860,7 +860,7 @@ def main():
                 "periodic_and_individual_steps": extras,
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
                 "gpu_launches": None}
-        lps = launches_per_step(w)
+        lps = launches_per_step(w, torch.cuda.get_device_properties(dev).multi_processor_count, prec == E.EVOL_FP32_MIXED)
         line["gpu_launches"] = (lps + args.kdk_steps * (lps + 3)) * args.steps if args.kdk_steps else lps * args.steps
         print(json.dumps(line), flush=True)
     if dist:
@@ -868,31 +868,46 @@ def main():
     return 0
 
 
-def launches_per_step(w):
-    """Kernels of ours per evol_step (the device chooses nothing here: both block shapes of a length
-    solve and both forms of a split walk are launched, one returns at once)."""
+# Sizes at which the library's launches change: direct ranking and one-kernel radix passes (csrc/tree.cu), leaf
+# lists of the length solves (csrc/lengths.cu), one-block scans (csrc/tree.cu).
+RANK_MAX, FUSED_MAX, LISTS_MIN, SCAN_ONE_MAX = 12288, 131072, 65536, 16384
+
+
+def launches_per_step(w, num_sms=152, mixed=False):
+    """Kernels of ours per evol_step.  Where the device chooses between two kernels both are launched and one
+    returns at once: the two block shapes of a length solve (open axes without the velocity divergence) and
+    the two forms of a walk that may be split."""
     p, n = w.params, w.n
     nsys = 1 if w.sys_offsets is None else len(w.sys_offsets) - 1
-    scan = lambda m: 1 if m <= 16384 else 3
+    scan = lambda m: 1 if m <= SCAN_ONE_MAX else 3
     digits = 1 if nsys > 1 else 0
     while nsys > 256 ** digits and nsys > 1:
         digits += 1
-    k = (1 if n <= 12288 or nsys > 1 else 2) + 1                       # bounding cube, keys
-    if n <= 12288:
+    k = (1 if n <= RANK_MAX or nsys > 1 else 2) + 1                    # bounding cube, keys
+    if n <= RANK_MAX:
         k += 1                                                         # direct ranking
     else:
-        one = 1 if n <= 131072 else 2 + scan(256 * ((n + 2047) // 2048))
+        one = 1 if n <= FUSED_MAX else 2 + scan(256 * ((n + 2047) // 2048))
         k += (8 + digits) * one + (2 if nsys > 1 else 0)               # passes; systems: ids, keys again
     k += 1 + 1 + scan(n) + 1 + 1 + 2                                   # permute, counts, nodes, links, moments
-    eps, h = bool(p.gravity and p.adaptive_softening), bool(p.sph and w.n_gas)
-    shared = eps and h and w.n_gas == n and p.n_nei_grav == p.n_nei_sph
-    if h and w.n_gas < n:
+    grav, sph = bool(p.gravity), bool(p.sph and w.n_gas)
+    eps = grav and bool(p.adaptive_softening)
+    shared = eps and sph and w.n_gas == n and p.n_nei_grav == p.n_nei_sph and not p.sph_scheme
+    if sph and w.n_gas < n:
         k += 2 + scan(n)                                               # gas lists
-    k += (int(eps) + int(h) - int(shared)) * (3 if n >= 65536 else 1)  # leaf lists and two shapes
+    curl = sph and bool(p.balsara or p.variable_alpha)
+
+    def solve(m, flow):                                                # leaf lists and one or two shapes
+        return 1 if m < LISTS_MIN else 2 if flow or p.periodic_mask else 3
+
+    k += (solve(n, curl and shared) if eps else 0) + (solve(w.n_gas, curl) if sph and not shared else 0)
     k += 1 + 1                                                         # operands, node lengths
-    ewald = p.gravity and p.periodic_mask
-    k += 0 if ewald else 1                                             # super-groups
-    k += 3 if (n <= 58368 and not ewald) else 1                        # walk
+    ewald = grav and bool(p.periodic_mask)
+    k += 0 if ewald or not (grav or sph) else 1                        # super-groups
+    diss = sph and bool(p.visc_form or p.balsara or p.variable_alpha or p.conduction)
+    blocks = 3 if (grav and sph) or (mixed and diss) else 4            # per SM, of four warps, of the split walk
+    split = not ewald and (n + 31) // 32 <= 4 * blocks * num_sms
+    k += 0 if not (grav or sph) else 3 if split else 1                 # walk
     return k + 1 + 2                                                   # results, diagnostics
 
 
