@@ -2,15 +2,17 @@
 // densitySPH, drhodr; Sect. 3.1 "gather" view with an enlarged search radius).
 //
 // Each particle i needs the particles within its search radius R_i = 2 L_i (1 + 0.1).  A block of
-// four warps takes 4 SUB consecutive particles in key order, SUB to a warp (evol_params.length_group;
-// by default chosen from their number, see group_size).  The block walks the tree once for all of
-// them, popping up to 128 nodes at a time and opening those whose particle box comes within a warp's
-// largest R_i of that warp's particle box; the particles of the leaves reached (the candidates) are
-// copied to shared memory, with the box of every 32 of them (a chunk).  Where the candidates do not
-// fit, the walk is repeated for halves of the particles.  A particle then tests the chunks against
-// its own ball and the candidates of the chunks that pass; those inside the ball are listed as
-// (distance, mass) pairs in shared memory.  A particle whose radius grows beyond its warp's, or
-// whose block's candidates did not fit even for single particles, walks the tree on its own.
+// NW = 4 or 8 warps (see Shape) takes NW SUB consecutive particles in key order, SUB to a warp (set by
+// evol_params.length_group, see warp_particles; by default chosen from their number, see group_size).
+// The block finds the leaves whose particle box comes within a warp's largest R_i of that warp's
+// particle box, from the leaf list of their super-group (k_leaf_lists) or by one walk of the tree
+// for all of them, popping up to 32 nodes a warp at a time; the particles of those leaves (the
+// candidates) are copied to shared memory, with the box of every 32 of them (a chunk).  Where the
+// candidates do not fit, the first of each warp's particles that should fit are taken and the others
+// wait for a later round.  A particle then tests the chunks against its own ball and the candidates of
+// the chunks that pass; those inside the ball are listed as distances with candidates or masses in
+// shared memory.  A particle whose radius grows beyond its warp's waits for a later round too, and one
+// whose block's candidates did not fit even for single particles walks the tree on its own.
 // On its list a particle solves
 //     F(L) = L^3 n(L) - eta^3 = 0,   n(L) = sum_j W(r_ij, L)  (self term included)
 // by Newton steps in L^3 kept inside a bisection bracket, gathering again when 2L leaves the gathered

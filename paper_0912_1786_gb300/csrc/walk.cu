@@ -43,7 +43,10 @@ constexpr int SG_GROUPS = EVOL_SG_GROUPS;   // groups per super-group (see k_sup
 // sums in d.wpart; k_walk_finish adds them up.  As many parts as give each warp of the grid about two items,
 // at most 16 (a part pays for the group's bounds and for partly filled batches): 1000 particles 0.25 ms whole
 // -> 0.11 (16 parts; 0.13 with 4, 0.12 with 32), 4096 particles 0.40 -> 0.16, 49,152 particles 1.11 -> 0.91 (2
-// parts; 0.97 with 4, 1.13 with 8).  With more groups than warps whole groups are as fast.
+// parts; 0.97 with 4, 1.13 with 8).  The line lies where every warp has a group; beyond it two parts are ahead
+// for a while yet (gravity + SPH, gas sphere, ms, whole groups / two parts: 60,000 particles 0.78 / 0.69,
+// 70,000 0.82 / 0.75, 80,000 0.85 / 0.86, 98,304 0.89 / 1.07; gravity alone, Plummer sphere, 80,000 0.74 /
+// 0.65, 131,072 1.04 / 0.94).
 constexpr int PART_MAX = 4;       // at most 2^4 parts
 
 __device__ __forceinline__ int walk_parts(int ngroups, int slots)
@@ -1480,7 +1483,7 @@ void launch_walk_pcd(evol_ctx *c, const evol_kparams &kp, bool mixed, bool check
 template <bool GRAV, bool SPH, bool EWALD>
 void launch_walk_pce(evol_ctx *c, const evol_kparams &kp, bool mixed, bool check)
 {
-    // the super-groups' top-of-tree walk first (one warp per block, 16 blocks per SM)
+    // the super-groups' top-of-tree walk first (one warp per block, 24 blocks per SM)
     const int nsg = (kp.n + 32 * SG_GROUPS - 1) / (32 * SG_GROUPS);
     if (!EWALD && kp.super && nsg > 0) k_super<GRAV, SPH, EWALD><<<c->num_sms * 24, 32, 0, c->stream>>>(c->d, kp, nsg);
     if constexpr (SPH) {
