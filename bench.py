@@ -644,7 +644,7 @@ def main():
         best, ms = E.evol_autotune(ctx, ds.particles, ds.params, ds.outputs, candidates=[12, 16, 24, 32, 48], reps=3)
         ds.params.leaf_size = best
         # then the length solves' group size at that leaf size
-        bg, msg = E.evol_autotune_length_group(ctx, ds.particles, ds.params, ds.outputs, candidates=[8, 16, 32],
+        bg, msg = E.evol_autotune_length_group(ctx, ds.particles, ds.params, ds.outputs, candidates=[8, 16],
                                                reps=3)
         ds.params.length_group = bg
         autotune = {"leaf_size": best, "median_ms_by_leaf": ms, "length_group": bg,
@@ -655,7 +655,7 @@ def main():
                                            which=E.EVOL_TUNE_LEAF_SIZE, candidates=[8, 12, 16, 24], reps=3)
         ds.params.leaf_size = best
         bg, msg = E.evol_autotune_batched(ctx, offsets, ds.particles, ds.params, ds.outputs,
-                                          which=E.EVOL_TUNE_LENGTH_GROUP, candidates=[8, 16, 32], reps=3)
+                                          which=E.EVOL_TUNE_LENGTH_GROUP, candidates=[8, 16], reps=3)
         ds.params.length_group = bg
         autotune = {"leaf_size": best, "median_ms_by_leaf": ms, "length_group": bg,
                     "median_ms_by_length_group": msg}

@@ -297,7 +297,9 @@ int evol_autotune(evol_ctx *ctx, evol_particles *p, const evol_params *prm, evol
 
 /* The same autotuner for the length solves' group size (prm->length_group), at the parameters
  * given (leaf size included): candidates in 1..32 (NULL: {4, 8, 16, 32}); *best receives the fastest,
- * ms_out (may be NULL) each candidate's median step time.  Same timing protocol as evol_autotune. */
+ * ms_out (may be NULL) each candidate's median step time.  Sizes that stand for the same number of
+ * particles per warp (see length_group) differ by the timing's noise only.  Same timing protocol as
+ * evol_autotune. */
 int evol_autotune_length_group(evol_ctx *ctx, evol_particles *p, const evol_params *prm, evol_outputs *out,
                                const int *candidates, int ncand, int reps, int *best, float *ms_out);
 
